@@ -5,17 +5,21 @@
 //
 // with x, xp in the 16-bit type (xp = X P from kd_apply_p, rounded by the caller), h()
 // the rounding of a centre to that type, fp32 accumulation.  Neither plane is expanded
-// in memory: each code becomes its 16-bit centre in registers and feeds an mma.sync B
-// fragment directly.
+// in memory.  This file holds the kernel for up to 16 batch rows (decode), the argument
+// checks and the entry points; more rows take kd_fold16_tc.cu, whose tcgen05 form decodes
+// every code once per 256 rows (7B layer: 101 us at 17 rows and 304 us at 512, where 16
+// rows at a time through this kernel took 201 us and 3.2 ms; at 16 rows and fewer the
+// clusters' set-up and barriers cost it more than they save: 105 us at 4 rows).
 //
-// Mapping.  mma.m16n8k16 with M = the batch rows (up to 16 per launch), N = 8 output
-// channels, K = 16 inputs.  A work item is a tile of 32 channels (four n-tiles) of one
-// matrix and one CTA; its four warps split the inputs into groups of 64 (four k-steps)
-// round-robin, each loading the next group's code words and inputs while it computes
-// the current one, then add their partial tiles in a fixed order (deterministic
-// results).  Items are numbered longest vectors first, so the hardware starts the long
-// ones first.  Launches of at most 8 batch rows skip the rows g + 8 of the A fragments
-// (fewer registers, more warps per SM).
+// Mapping.  mma.m16n8k16 with M = the batch rows, N = 8 output channels, K = 16 inputs: each
+// code becomes its 16-bit centre in registers (kd_dec16.cuh) and feeds a B fragment
+// directly.  A work item is a tile of 32 channels (four n-tiles) of one matrix and one CTA;
+// its warps split the inputs into groups of 64 (four k-steps) round-robin, each loading the
+// next group's code words and inputs while it computes the current one, then add their
+// partial tiles in a fixed order (deterministic results).  Items are numbered longest
+// vectors first, so the hardware starts the long ones first.  Launches of at most 8 batch
+// rows skip the rows g + 8 of the A fragments (fewer registers).  Bound by the decode on
+// the ALU pipe (62 % busy at 4 rows, 7B layer, 78 us).
 //
 // K order inside a group of 64 inputs.  The product is a sum over inputs, so A and B
 // may enumerate them in any common order.  In k-step j the lanes with t = lane % 4
@@ -24,22 +28,19 @@
 // consecutive inputs of rows g and g + 8 (g = lane / 4: two 16-byte loads per row), and
 // its B fragments are code word t of the group (inputs 16 t .. 16 t + 15) of its
 // channel: byte j of that word holds the four codes of k-step j.
-//
-// Decoding.  The four 16-bit centres of a channel are kept as two words, L (their low
-// bytes) and H (their high bytes).  For two codes q0, q1 one byte permute with the
-// selector nibbles (q0, q0 + 4, q1, q1 + 4) yields the pair (c[q0], c[q1]); the
-// selectors of two k-steps are formed together from one shifted code word.
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "kashin.h"
+#include "kd_dec16.cuh"
+#include "kd_fold16.h"
 
 namespace kd {
 namespace {
 
-constexpr int kF16Warps = 4;
-constexpr int kF16Threads = 32 * kF16Warps;
+// warps of a CTA, which split the inputs: eight up to 8 batch rows (two CTAs per SM; with
+// four and four, the last items of a 7B layer ran on a third of the SMs: 78 against 86 us
+// per layer at 4 rows), four beyond (the upper rows' fragments need the registers)
+__host__ __device__ constexpr int f16_warps(bool hi) { return hi ? 4 : 8; }
 constexpr int kF16Rows = 16;  // batch rows per launch (the mma's M)
 constexpr int kF16Tile = 32;  // output channels per work item (four n-tiles)
 constexpr int kRedStride = kF16Tile + 1;
@@ -61,6 +62,7 @@ struct Fold16Params {
   int count;
   int rows;  // batch rows of this launch (<= 16)
   int64_t items;
+  DecodeMul mul;
   Fold16Mat mat[KD_MAX_BATCH];
 };
 
@@ -79,32 +81,6 @@ __device__ __forceinline__ void mma_16(float (&d)[4], uint32_t a0, uint32_t a1, 
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
   }
-}
-
-// a centre rounded (nearest, ties to even) to the activations' 16-bit type, as bits
-template <bool BF>
-__device__ __forceinline__ uint32_t bits16(float c) {
-  if constexpr (BF) return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(c));
-  else return (uint32_t)__half_as_ushort(__float2half_rn(c));
-}
-
-// Byte selectors for the code nibbles at bits 0..3 (low half) and 16..19 (high half) of
-// t: nibble v = q0 | q1 << 2 gives the selector nibbles (q0, q0 + 4, q1, q1 + 4).
-__device__ __forceinline__ uint32_t selectors(uint32_t t) {
-  // q0 to bits 0-1, q1 to bits 8-9 (and 16-17, 24-25): one mask, one shift, one multiplex
-  const uint32_t u = t & 0x000F000Fu;
-  const uint32_t x = (u & 0x00C300C3u) | ((u << 6) & ~0x00C300C3u);
-  return x * 0x11u + 0x40404040u;
-}
-
-// The 16-bit centres of one channel as (low bytes, high bytes), zero past m.
-template <bool BF>
-__device__ __forceinline__ uint2 centre_bytes(const float* centres, int64_t j, bool ok) {
-  if (!ok) return make_uint2(0u, 0u);
-  const float4 c = __ldg(reinterpret_cast<const float4*>(centres) + j);
-  const uint32_t p01 = bits16<BF>(c.x) | (bits16<BF>(c.y) << 16);
-  const uint32_t p23 = bits16<BF>(c.z) | (bits16<BF>(c.w) << 16);
-  return make_uint2(__byte_perm(p01, p23, 0x6420u), __byte_perm(p01, p23, 0x7531u));
 }
 
 // A lane's 16 fp16 inputs of one row at i0 .. i0 + 15 as 8 pairs, zero past n or for a
@@ -131,8 +107,9 @@ __device__ __forceinline__ void load_row16(uint32_t (&r)[8], const unsigned shor
 }
 
 template <bool HI, bool BF>
-__global__ void __launch_bounds__(kF16Threads, HI ? 3 : 4) fold16_kernel(const __grid_constant__ Fold16Params p) {
-  __shared__ float red[kF16Warps][kF16Rows][kRedStride];
+__global__ void __launch_bounds__(32 * f16_warps(HI), HI ? 3 : 2) fold16_kernel(const __grid_constant__ Fold16Params p) {
+  constexpr int W = f16_warps(HI);
+  __shared__ float red[W][kF16Rows][kRedStride];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -191,36 +168,30 @@ __global__ void __launch_bounds__(kF16Threads, HI ? 3 : 4) fold16_kernel(const _
       }
     };
     if (warp < groups) fetch(warp);
-    for (int64_t gi = warp; gi < groups; gi += kF16Warps) {
+    for (int64_t gi = warp; gi < groups; gi += W) {
       uint32_t cwu[4], cwv[4], cax[8], caxh[8], cap[8], caph[8];
 #pragma unroll
       for (int k = 0; k < 4; ++k) { cwu[k] = wu[k]; cwv[k] = wv[k]; }
 #pragma unroll
       for (int k = 0; k < 8; ++k) { cax[k] = ax[k]; caxh[k] = axh[k]; cap[k] = ap[k]; caph[k] = aph[k]; }
-      if (gi + kF16Warps < groups) fetch(gi + kF16Warps);
+      if (gi + W < groups) fetch(gi + W);
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt) {
-        // k-steps (0, 2) from nibbles at bits (0, 16) and (4, 20); (1, 3) from (8, 24), (12, 28)
-        const uint32_t su0 = selectors(cwu[nt]), su1 = selectors(cwu[nt] >> 4);
-        const uint32_t su2 = selectors(cwu[nt] >> 8), su3 = selectors(cwu[nt] >> 12);
-        const uint32_t sv0 = selectors(cwv[nt]), sv1 = selectors(cwv[nt] >> 4);
-        const uint32_t sv2 = selectors(cwv[nt] >> 8), sv3 = selectors(cwv[nt] >> 12);
+        // pairs (4 j, 4 j + 1) and (4 j + 2, 4 j + 3) of the word are k-step j's B fragment
+        uint4 ul, uh, vl, vh;
+        decode_word(cwu[nt], cu[nt], p.mul, ul, uh);
+        decode_word(cwv[nt], cv[nt], p.mul, vl, vh);
+        const uint32_t bu[8] = {ul.x, ul.y, ul.z, ul.w, uh.x, uh.y, uh.z, uh.w};
+        const uint32_t bv[8] = {vl.x, vl.y, vl.z, vl.w, vh.x, vh.y, vh.z, vh.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const uint32_t s0u = (j & 1) ? su2 : su0, s1u = (j & 1) ? su3 : su1;
-          const uint32_t s0v = (j & 1) ? sv2 : sv0, s1v = (j & 1) ? sv3 : sv1;
-          const int sh = (j & 2) ? 16 : 0;
-          const uint32_t bu0 = __byte_perm(cu[nt].x, cu[nt].y, s0u >> sh);
-          const uint32_t bu1 = __byte_perm(cu[nt].x, cu[nt].y, s1u >> sh);
-          const uint32_t bv0 = __byte_perm(cv[nt].x, cv[nt].y, s0v >> sh);
-          const uint32_t bv1 = __byte_perm(cv[nt].x, cv[nt].y, s1v >> sh);
-          mma_16<BF>(acc[nt], cax[2 * j], caxh[2 * j], cax[2 * j + 1], caxh[2 * j + 1], bu0, bu1);
-          mma_16<BF>(acc[nt], cap[2 * j], caph[2 * j], cap[2 * j + 1], caph[2 * j + 1], bv0, bv1);
+          mma_16<BF>(acc[nt], cax[2 * j], caxh[2 * j], cax[2 * j + 1], caxh[2 * j + 1], bu[2 * j], bu[2 * j + 1]);
+          mma_16<BF>(acc[nt], cap[2 * j], caph[2 * j], cap[2 * j + 1], caph[2 * j + 1], bv[2 * j], bv[2 * j + 1]);
         }
       }
     }
 
-    // partial tiles of the four warps, added in warp order
+    // partial tiles of the warps, added in warp order
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
       red[warp][g][8 * nt + 2 * t] = acc[nt][0];
@@ -229,12 +200,12 @@ __global__ void __launch_bounds__(kF16Threads, HI ? 3 : 4) fold16_kernel(const _
       red[warp][g + 8][8 * nt + 2 * t + 1] = acc[nt][3];
     }
     __syncthreads();
-    for (int o = threadIdx.x; o < kF16Rows * kF16Tile; o += kF16Threads) {
+    for (int o = threadIdx.x; o < kF16Rows * kF16Tile; o += 32 * W) {
       const int r = o / kF16Tile, c = o % kF16Tile;
       if (r < p.rows && c0 + c < a.m) {
         float s = red[0][r][c];
 #pragma unroll
-        for (int w = 1; w < kF16Warps; ++w) s = __fadd_rn(s, red[w][r][c]);
+        for (int w = 1; w < W; ++w) s = __fadd_rn(s, red[w][r][c]);
         a.y[(int64_t)r * a.ldy + c0 + c] = s;
       }
     }
@@ -270,55 +241,53 @@ kd_status fold16_run(const kd_fold_mat_f16* mats, int count, int64_t batch, void
   for (int i = 0; i < count; ++i) work += mats[i].m;
   if (batch == 0 || work == 0) return KD_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // batch rows sixteen at a time (the mma's M): each launch reads the code planes once
-  for (int64_t b0 = 0; b0 < batch; b0 += kF16Rows) {
-    Fold16Params p;
-    p.count = count;
-    p.rows = (int)(batch - b0 < kF16Rows ? batch - b0 : kF16Rows);
-    // work items numbered longest vectors first, so that the long items of a layer are
-    // not the last ones started
-    int order[KD_MAX_BATCH];
-    for (int i = 0; i < count; ++i) order[i] = i;
-    for (int i = 1; i < count; ++i)
-      for (int k = i; k > 0 && mats[order[k]].n > mats[order[k - 1]].n; --k) {
-        const int tmp = order[k];
-        order[k] = order[k - 1];
-        order[k - 1] = tmp;
-      }
-    int64_t items = 0;
-    for (int i = 0; i < count; ++i) {
-      const kd_fold_mat_f16& a = mats[order[i]];
-      Fold16Mat& f = p.mat[i];
-      f.codes_u = a.codes_u;
-      f.codes_v = a.codes_v;
-      f.centres_u = a.centres_u;
-      f.centres_v = a.centres_v;
-      f.x = static_cast<const unsigned short*>(a.x) + b0 * a.ldx;
-      f.xp = static_cast<const unsigned short*>(a.xp) + b0 * a.ldx;
-      f.y = a.y + b0 * a.ldy;
-      f.n = a.n;
-      f.m = a.m;
-      f.words = (a.n + 15) / 16;
-      f.ldx = a.ldx;
-      f.ldy = a.ldy;
-      f.item0 = items;
-      f.vec = aligned16(f.x, 16) && aligned16(f.xp, 16) && a.ldx % 8 == 0;
-      items += (a.m + kF16Tile - 1) / kF16Tile;
+  if (batch > kF16Rows) return fold16_tc_run(mats, count, batch, s, bf);
+  // one launch reads the code planes once
+  Fold16Params p;
+  p.count = count;
+  p.rows = (int)batch;
+  // work items numbered longest vectors first, so that the long items of a layer are
+  // not the last ones started
+  int order[KD_MAX_BATCH];
+  for (int i = 0; i < count; ++i) order[i] = i;
+  for (int i = 1; i < count; ++i)
+    for (int k = i; k > 0 && mats[order[k]].n > mats[order[k - 1]].n; --k) {
+      const int tmp = order[k];
+      order[k] = order[k - 1];
+      order[k - 1] = tmp;
     }
-    p.items = items;
-    if (items == 0) continue;
-    // one CTA per work item (the grid-stride loop covers grids past 2^30 items)
-    const int64_t grid = items < (int64_t)1 << 30 ? items : (int64_t)1 << 30;
-    const unsigned gr = (unsigned)grid;
-    if (bf) {
-      if (p.rows > 8) fold16_kernel<true, true><<<gr, kF16Threads, 0, s>>>(p);
-      else fold16_kernel<false, true><<<gr, kF16Threads, 0, s>>>(p);
-    } else {
-      if (p.rows > 8) fold16_kernel<true, false><<<gr, kF16Threads, 0, s>>>(p);
-      else fold16_kernel<false, false><<<gr, kF16Threads, 0, s>>>(p);
-    }
-    if (cudaGetLastError() != cudaSuccess) return KD_ERR_CUDA;
+  int64_t items = 0;
+  for (int i = 0; i < count; ++i) {
+    const kd_fold_mat_f16& a = mats[order[i]];
+    Fold16Mat& f = p.mat[i];
+    f.codes_u = a.codes_u;
+    f.codes_v = a.codes_v;
+    f.centres_u = a.centres_u;
+    f.centres_v = a.centres_v;
+    f.x = static_cast<const unsigned short*>(a.x);
+    f.xp = static_cast<const unsigned short*>(a.xp);
+    f.y = a.y;
+    f.n = a.n;
+    f.m = a.m;
+    f.words = (a.n + 15) / 16;
+    f.ldx = a.ldx;
+    f.ldy = a.ldy;
+    f.item0 = items;
+    f.vec = aligned16(f.x, 16) && aligned16(f.xp, 16) && a.ldx % 8 == 0;
+    items += (a.m + kF16Tile - 1) / kF16Tile;
   }
+  p.items = items;
+  // one CTA per work item (the grid-stride loop covers grids past 2^30 items)
+  const int64_t grid = items < (int64_t)1 << 30 ? items : (int64_t)1 << 30;
+  const unsigned gr = (unsigned)grid;
+  if (bf) {
+    if (p.rows > 8) fold16_kernel<true, true><<<gr, 32 * f16_warps(true), 0, s>>>(p);
+    else fold16_kernel<false, true><<<gr, 32 * f16_warps(false), 0, s>>>(p);
+  } else {
+    if (p.rows > 8) fold16_kernel<true, false><<<gr, 32 * f16_warps(true), 0, s>>>(p);
+    else fold16_kernel<false, false><<<gr, 32 * f16_warps(false), 0, s>>>(p);
+  }
+  if (cudaGetLastError() != cudaSuccess) return KD_ERR_CUDA;
   return KD_OK;
 }
 

@@ -498,7 +498,7 @@ def matmul_2bit_f16(dec: "Decomposed", x, xp, out=None, stream=None):
 
 def matmul_2bit_f16_batch(decs, xs, xps, outs=None, stream=None):
     """kd_matmul_2bit_f16_batch (or _bf16_batch, for bf16 inputs): ``Y_i = X_i W_hat_i^T``
-    for several matrices, 16-bit inputs of one type and batch size, one launch per 16 rows."""
+    for several matrices, 16-bit inputs of one type and batch size, in one launch."""
     torch = _torch()
     dt = xs[0].dtype
     if dt not in (torch.float16, torch.bfloat16):
