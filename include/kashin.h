@@ -373,8 +373,9 @@ kd_status kd_measure_fp32_peak(double* tflops, void* stream);
  *   xp                 device fp32, the same rows times P (kd_apply_p with the matrix's
  *                      sign seed on the rows of X), same layout and ldx.
  *   y                  device fp32, batch rows of m outputs, row r at y + r*ldy (ldy >= m).
- * Every code word is read once per group of up to two batch rows; accumulation is
- * fp32 in a fixed order (deterministic).  Errors: KD_ERR_INVALID_ARG (sizes, null or
+ * Every code word is read once per group of up to 16 batch rows; nothing is rounded below
+ * fp32, and the sums run in a fixed order (deterministic).  A wait inside the kernel that
+ * exceeds its time limit leaves NaN in the outputs it concerns.  Errors: KD_ERR_INVALID_ARG (sizes, null or
  * unaligned pointers when m > 0 and batch > 0), KD_ERR_CUDA (launch).  m == 0 or
  * batch == 0 enqueues nothing. */
 kd_status kd_matmul_2bit(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,
@@ -407,9 +408,9 @@ kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, int64_t batch
  *   y[r*ldy + j] = sum_i h(centres_u[j][code_u(j,i)]) x[r*ldx + i]
  *                + sum_i h(centres_v[j][code_v(j,i)]) xp[r*ldx + i],   r < batch, j < m,
  * where x and xp are fp16 (IEEE binary16) and h() rounds a centre to fp16 (nearest,
- * ties to even); products are exact and the sums are fp32.  This
- * is Y = X W_hat^T in the precision of a dense fp16 layer: the activations and the
- * weights' values are fp16, nothing else is rounded.
+ * ties to even); products are exact and the sums are fp32.  This is Y = X W_hat^T in the
+ * precision of a dense fp16 layer: the activations and the weights' values are fp16, nothing
+ * else is rounded.
  *   codes_u, codes_v, centres_u, centres_v, n, m, batch, y, ldy as in kd_matmul_2bit.
  *   x, xp   device fp16, batch rows of n inputs, row r at x + r*ldx (ldx >= n);
  *           xp holds the rows of X P (kd_apply_p, rounded to fp16 by the caller).
@@ -419,16 +420,14 @@ kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, int64_t batch
  * a zero input by a centre.  Every code word is read once for up to 16 batch rows, and
  * once per block of up to 256 rows beyond; the sums run in a fixed order that depends on
  * the batch size (deterministic).  A wait inside the kernel that exceeds its time limit
- * leaves NaN in the outputs it concerns.  Errors and empty calls as
- * kd_matmul_2bit. */
+ * leaves NaN in the outputs it concerns.  Errors and empty calls as kd_matmul_2bit. */
 kd_status kd_matmul_2bit_f16(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,
                              const float* centres_v, int64_t n, int64_t m, const void* x, const void* xp,
                              int64_t batch, int64_t ldx, float* y, int64_t ldy, void* stream);
 
 /* kd_matmul_2bit_f16 for several matrices in one launch (one more for matrices whose rows
- * are not 16-byte aligned); each
- * descriptor as kd_matmul_2bit_f16's arguments.  mats is a HOST array of 1 <= count <=
- * KD_MAX_BATCH descriptors.  Results equal kd_matmul_2bit_f16's per matrix, bit for bit.
+ * are not 16-byte aligned); each descriptor as kd_matmul_2bit_f16's arguments.  mats is a
+ * HOST array of 1 <= count <= KD_MAX_BATCH descriptors.  Results equal kd_matmul_2bit_f16's per matrix, bit for bit.
  * Errors as kd_matmul_2bit_batch. */
 typedef struct kd_fold_mat_f16 {
   const uint32_t* codes_u;
@@ -448,8 +447,8 @@ kd_status kd_matmul_2bit_f16_batch(const kd_fold_mat_f16* mats, int count, int64
 
 /* kd_matmul_2bit_f16 and its batched form for bf16 activations: x and xp are bf16, each
  * centre is rounded to bf16 (nearest, ties to even), products are exact and sums
- * fp32.  Arguments, layouts, alignment and errors as the fp16
- * calls (the descriptor struct is shared). */
+ * fp32.  Arguments, layouts, alignment and errors as the fp16 calls (the descriptor struct
+ * is shared). */
 kd_status kd_matmul_2bit_bf16(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,
                               const float* centres_v, int64_t n, int64_t m, const void* x, const void* xp,
                               int64_t batch, int64_t ldx, float* y, int64_t ldy, void* stream);

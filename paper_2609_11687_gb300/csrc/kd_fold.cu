@@ -7,19 +7,24 @@
 // with xp = X P from kd_apply_p.  Neither U_q nor V_q is expanded: every weight costs
 // its 2-bit code in each plane (0.5 byte per weight in all), read once from HBM.
 //
+// This file holds the argument checks, the entry points and the kernel for one batch row;
+// two rows and more take kd_fold_tc.cu, on the tensor cores, 16 rows in one pass over the
+// codes (7B layer: 116 us at 2 rows and 126 at 16, where this kernel, two rows at a time,
+// took 121 and 970; at one row it takes 85).
+//
 // Mapping.  One launch serves up to KD_MAX_BATCH matrices (a layer): persistent CTAs
-// of eight warps walk the work items (matrix, tile of RT = 16 / B output channels).
+// of eight warps walk the work items (matrix, tile of RT = 16 output channels).
 // Per item each warp takes slices of 32 consecutive code words (512 inputs): it loads
 // its lane's 16 inputs of x and xp (L2-resident, shared by every item of the matrix)
 // into registers, then the code words of all RT channels of the tile (one coalesced
 // word per channel, plane and lane, all in flight together).  Two codes at a time (4
 // bits) index a per-channel table of the 16 centre pairs (c[q0], c[q1]) in shared
-// memory: one 64-bit shared load and one packed FP32x2 FMA per two weights, plane
-// and batch row.  The lanes' and warps' partial sums are added in a fixed order
+// memory: one 64-bit shared load and one packed FP32x2 FMA per two weights and plane.  The lanes' and warps' partial sums are added in a fixed order
 // (deterministic results).
 #include <cuda_runtime.h>
 
 #include "kashin.h"
+#include "kd_fold_tc.h"
 
 namespace kd {
 namespace {
@@ -35,29 +40,20 @@ struct FoldMat {
   const float* x;
   const float* xp;
   float* y;
-  int64_t n, m, words, ldx, ldy;
+  int64_t n, m, words;
   int64_t tile0;  // first work item of this matrix
-  int vec;        // x and xp 16-byte aligned with ldx a multiple of 4: 128-bit input loads
+  int vec;        // x and xp 16-byte aligned: 128-bit input loads
 };
 
 struct FoldParams {
   int count;
-  int rows;        // batch rows of this launch (<= B)
   int64_t items;   // work items of all matrices
   FoldMat mat[KD_MAX_BATCH];
 };
 
-// RT x B = 16 partial sums per lane
-template <int B>
-struct FoldTile {
-  static constexpr int RT = 16 / B;
-};
+constexpr int RT = 16;  // output channels per work item: partial sums per lane
 
-template <int B>
 __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_constant__ FoldParams p) {
-  constexpr int RT = FoldTile<B>::RT;
-  constexpr int K = RT * B;  // partial sums per lane
-  static_assert(K == 16, "the reduction scatters 16 values per lane");
   __shared__ float2 tab[2 * RT * 16];
   __shared__ float red[kFoldWarps * 16];
   const int lane = threadIdx.x & 31;
@@ -84,11 +80,9 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
     }
     __syncthreads();
 
-    float2 acc[RT][B];
+    float2 acc[RT];
 #pragma unroll
-    for (int r = 0; r < RT; ++r)
-#pragma unroll
-      for (int b = 0; b < B; ++b) acc[r][b] = make_float2(0.f, 0.f);
+    for (int r = 0; r < RT; ++r) acc[r] = make_float2(0.f, 0.f);
 
     const int64_t nslices = (a.words + 31) / 32;
     for (int64_t s = warp; s < nslices; s += kFoldWarps) {
@@ -101,34 +95,26 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
         cu[r] = ok ? __ldg(a.codes_u + (j0 + r) * a.words + wi) : 0u;
         cv[r] = ok ? __ldg(a.codes_v + (j0 + r) * a.words + wi) : 0u;
       }
-      // this lane's 16 inputs of x and xp per batch row (zero past n and past the rows):
-      // four 128-bit loads each when the whole word lies inside aligned rows
-      float2 xv[B][8], pv[B][8];
-      {
-        const bool vec = a.vec && 16 * wi + 16 <= a.n;
+      // this lane's 16 inputs of x and xp (zero past n): four 128-bit loads each when the
+      // whole word lies inside aligned rows
+      float2 xv[8], pv[8];
+      if (valid && a.vec && 16 * wi + 16 <= a.n) {
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-          const bool live = valid && b < p.rows;
-          const int64_t o0 = (int64_t)b * a.ldx + 16 * wi;
-          if (vec && live) {
+        for (int k = 0; k < 8; k += 2) {
+          const float4 u = __ldg(reinterpret_cast<const float4*>(a.x + 16 * wi + 2 * k));
+          const float4 w = __ldg(reinterpret_cast<const float4*>(a.xp + 16 * wi + 2 * k));
+          xv[k] = make_float2(u.x, u.y);
+          xv[k + 1] = make_float2(u.z, u.w);
+          pv[k] = make_float2(w.x, w.y);
+          pv[k + 1] = make_float2(w.z, w.w);
+        }
+      } else {
 #pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-              const float4 u = __ldg(reinterpret_cast<const float4*>(a.x + o0 + 2 * k));
-              const float4 w = __ldg(reinterpret_cast<const float4*>(a.xp + o0 + 2 * k));
-              xv[b][k] = make_float2(u.x, u.y);
-              xv[b][k + 1] = make_float2(u.z, u.w);
-              pv[b][k] = make_float2(w.x, w.y);
-              pv[b][k + 1] = make_float2(w.z, w.w);
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int64_t i = 16 * wi + 2 * k;
-              const bool i0 = live && i < a.n, i1 = live && i + 1 < a.n;
-              xv[b][k] = make_float2(i0 ? __ldg(a.x + o0 + 2 * k) : 0.f, i1 ? __ldg(a.x + o0 + 2 * k + 1) : 0.f);
-              pv[b][k] = make_float2(i0 ? __ldg(a.xp + o0 + 2 * k) : 0.f, i1 ? __ldg(a.xp + o0 + 2 * k + 1) : 0.f);
-            }
-          }
+        for (int k = 0; k < 8; ++k) {
+          const int64_t i = 16 * wi + 2 * k;
+          const bool i0 = valid && i < a.n, i1 = valid && i + 1 < a.n;
+          xv[k] = make_float2(i0 ? __ldg(a.x + i) : 0.f, i1 ? __ldg(a.x + i + 1) : 0.f);
+          pv[k] = make_float2(i0 ? __ldg(a.xp + i) : 0.f, i1 ? __ldg(a.xp + i + 1) : 0.f);
         }
       }
 #pragma unroll
@@ -137,24 +123,19 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
         for (int k = 0; k < 8; ++k) {
           const float2 tu = tab[r * 16 + ((cu[r] >> (4 * k)) & 15u)];
           const float2 tv = tab[(RT + r) * 16 + ((cv[r] >> (4 * k)) & 15u)];
-#pragma unroll
-          for (int b = 0; b < B; ++b) {
-            acc[r][b] = __ffma2_rn(tu, xv[b][k], acc[r][b]);
-            acc[r][b] = __ffma2_rn(tv, pv[b][k], acc[r][b]);
-          }
+          acc[r] = __ffma2_rn(tu, xv[k], acc[r]);
+          acc[r] = __ffma2_rn(tv, pv[k], acc[r]);
         }
       }
     }
 
     // lane sums, then a butterfly reduce-scatter: lane l ends with its warp's total of
-    // value l % 16 (value index r * B + b)
-    float v[K];
+    // channel l % 16
+    float v[RT];
 #pragma unroll
-    for (int r = 0; r < RT; ++r)
+    for (int r = 0; r < RT; ++r) v[r] = __fadd_rn(acc[r].x, acc[r].y);
 #pragma unroll
-      for (int b = 0; b < B; ++b) v[r * B + b] = __fadd_rn(acc[r][b].x, acc[r][b].y);
-#pragma unroll
-    for (int k = K / 2; k >= 1; k >>= 1) {
+    for (int k = RT / 2; k >= 1; k >>= 1) {
 #pragma unroll
       for (int i = 0; i < k; ++i) {
         const bool hi = (lane & k) != 0;
@@ -164,29 +145,27 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
       }
     }
     v[0] = __fadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], 16));
-    if (lane < K) red[warp * 16 + lane] = v[0];
+    if (lane < RT) red[warp * 16 + lane] = v[0];
     __syncthreads();
-    if (threadIdx.x < K) {
+    if (threadIdx.x < RT) {
       float t = red[threadIdx.x];
 #pragma unroll
       for (int w = 1; w < kFoldWarps; ++w) t = __fadd_rn(t, red[w * 16 + threadIdx.x]);
-      const int r = threadIdx.x / B, b = threadIdx.x % B;
-      if (j0 + r < a.m && b < p.rows) a.y[(int64_t)b * a.ldy + j0 + r] = t;
+      if (j0 + threadIdx.x < a.m) a.y[j0 + threadIdx.x] = t;
     }
   }
 }
 
-template <int B>
 cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
   int dev = 0, sms = 0, per = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fold_kernel<B>, kFoldThreads, 0)) != cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fold_kernel, kFoldThreads, 0)) != cudaSuccess)
     return e;
   if (per < 1) return cudaErrorInvalidConfiguration;
   const int64_t grid = p.items < (int64_t)per * sms ? p.items : (int64_t)per * sms;
-  fold_kernel<B><<<(unsigned)grid, kFoldThreads, 0, s>>>(p);
+  fold_kernel<<<(unsigned)grid, kFoldThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -219,40 +198,29 @@ extern "C" kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, in
   }
   if (batch == 0) return KD_OK;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // batch rows two (or one) at a time: each launch reads the code planes once
-  for (int64_t b0 = 0; b0 < batch;) {
-    const int rows = batch - b0 >= 2 ? 2 : 1;
-    const int rt = rows == 2 ? kd::FoldTile<2>::RT : kd::FoldTile<1>::RT;
-    kd::FoldParams p;
-    p.count = count;
-    p.rows = rows;
-    int64_t items = 0;
-    for (int i = 0; i < count; ++i) {
-      const kd_fold_mat& a = mats[i];
-      kd::FoldMat& f = p.mat[i];
-      f.codes_u = a.codes_u;
-      f.codes_v = a.codes_v;
-      f.centres_u = a.centres_u;
-      f.centres_v = a.centres_v;
-      f.x = a.x + b0 * a.ldx;
-      f.xp = a.xp + b0 * a.ldx;
-      f.y = a.y + b0 * a.ldy;
-      f.n = a.n;
-      f.m = a.m;
-      f.words = (a.n + 15) / 16;
-      f.ldx = a.ldx;
-      f.ldy = a.ldy;
-      f.tile0 = items;
-      f.vec = kd::aligned(f.x, 16) && kd::aligned(f.xp, 16) && a.ldx % 4 == 0;
-      items += (a.m + rt - 1) / rt;
-    }
-    p.items = items;
-    if (items > 0) {
-      const cudaError_t e = rows == 2 ? kd::launch_fold<2>(p, s) : kd::launch_fold<1>(p, s);
-      if (e != cudaSuccess) return KD_ERR_CUDA;
-    }
-    b0 += rows;
+  if (batch > 1) return kd::fold_tc_run(mats, count, batch, s);
+  kd::FoldParams p;
+  p.count = count;
+  int64_t items = 0;
+  for (int i = 0; i < count; ++i) {
+    const kd_fold_mat& a = mats[i];
+    kd::FoldMat& f = p.mat[i];
+    f.codes_u = a.codes_u;
+    f.codes_v = a.codes_v;
+    f.centres_u = a.centres_u;
+    f.centres_v = a.centres_v;
+    f.x = a.x;
+    f.xp = a.xp;
+    f.y = a.y;
+    f.n = a.n;
+    f.m = a.m;
+    f.words = (a.n + 15) / 16;
+    f.tile0 = items;
+    f.vec = kd::aligned(f.x, 16) && kd::aligned(f.xp, 16);
+    items += (a.m + kd::RT - 1) / kd::RT;
   }
+  p.items = items;
+  if (items > 0 && kd::launch_fold(p, s) != cudaSuccess) return KD_ERR_CUDA;
   return KD_OK;
 }
 

@@ -7,9 +7,8 @@
 // the rounding of a centre to that type, fp32 accumulation.  Neither plane is expanded
 // in memory.  This file holds the kernel for up to 16 batch rows (decode), the argument
 // checks and the entry points; more rows take kd_fold16_tc.cu, whose tcgen05 form decodes
-// every code once per 256 rows (7B layer: 101 us at 17 rows and 304 us at 512, where 16
-// rows at a time through this kernel took 201 us and 3.2 ms; at 16 rows and fewer the
-// clusters' set-up and barriers cost it more than they save: 105 us at 4 rows).
+// every code once per 256 rows (7B layer: 88 us at 17 rows and 291 us at 512, where 16
+// rows at a time through this kernel took 195 us and 3.2 ms).
 //
 // Mapping.  mma.m16n8k16 with M = the batch rows, N = 8 output channels, K = 16 inputs: each
 // code becomes its 16-bit centre in registers (kd_dec16.cuh) and feeds a B fragment

@@ -6,17 +6,19 @@
 // K = the inputs: u plane against x, then v plane against xp.  A CTA owns one tile of 128
 // channels and (part of) K, cut into units of 128 inputs, each two stages of 64:
 //  * two groups of eight warps decode the codes, every other unit each: a thread reads 16
-//    bytes of its channel's code row, turns them into 64 16-bit centres and writes its
-//    128-byte row of the A tile (sixteen warps: with eight, two per scheduler, the decode's
-//    dependent chains left the MMAs waiting at 256 rows);
+//    bytes of its channel's code row, turns them into 64 16-bit centres and writes them to
+//    its TMEM lane (sixteen warps: with eight, two per scheduler, the decode's dependent
+//    chains left the MMAs waiting at 256 rows.  A in TMEM: through shared memory its writes
+//    and reads, with B's, filled the bandwidth, and 512 rows took 304 us);
 //  * one thread loads the B tiles (64 inputs of every batch row) by TMA, zero past the last
 //    input and the last row; where the rows are not 16-byte aligned the decoding threads
 //    fill them instead, element by element;
 //  * one thread issues the MMAs.
-// The accumulators live in TMEM in two buffers.  Every kChunk units the running sum moves
-// to the other buffer and the decoding warps add the finished one to fp32 registers: the
-// tensor core adds with less than fp32's rounding, so its chains are kept at 64 steps
-// (half of what a warp of the mma.sync kernel this one replaced had at n = 4096).
+// The accumulators live in TMEM, in two buffers where they fit beside the A slots (up to 128
+// rows).  Every kChunk units the decoding warps add the finished sums to fp32 registers,
+// while the next ones go to the other buffer: the tensor core adds with less than fp32's
+// rounding, so its chains are kept at 64 steps (half of what a warp of the mma.sync kernel
+// had at n = 4096).
 //
 // Split of K.  The decode of 128 x 128 weights costs 370 SM cycles of the ALU pipe at least,
 // the MMAs 4 N, so up to about 90 rows the time is the decode's and every SM has to take its
@@ -25,8 +27,8 @@
 // in rank order.  The split follows from the batch alone, so a matrix gives the same bits
 // alone and in a batched call.
 //
-// Measured (7B layer): 101 / 116 / 135 / 171 / 304 us at 17 / 64 / 128 / 256 / 512 rows; at
-// 512 rows that is 1.36 PFLOP/s, 70 % of the measured bf16 rate.  The MMA thread branches on
+// Measured (7B layer): 88 / 98 / 129 / 159 / 291 us at 17 / 64 / 128 / 256 / 512 rows; at 512
+// rows that is 1.43 PFLOP/s, 74 % of the measured bf16 rate.  The MMA thread branches on
 // elect.sync (kd_tc.cuh): with a lane test instead, every tcgen05 instruction cost a loop
 // over the lanes and 512 rows took 422 us.
 #include <cuda_runtime.h>
@@ -45,9 +47,9 @@ constexpr int kUnitK = 128;       // inputs per unit: two stages
 constexpr int kChunk = 8;         // units per TMEM accumulation (64 MMA steps)
 constexpr int kDecWarps = 16;     // decoding warps: two groups of eight
 constexpr int kThreads = 32 * (kDecWarps + 2);  // + the TMA warp and the MMA warp
-constexpr int kMaxA = 3;          // A slots (units), at most
+constexpr int kMaxA = 4;          // A slots (units), at most
 constexpr int kMaxB = 8;          // B slots, at most
-constexpr int kABytes = 2 * kTile * 128;  // one unit of A
+constexpr int kACols = 64;        // TMEM columns of one unit of A
 
 struct alignas(128) FoldTcMat {
   CUtensorMap map_x, map_xp;  // launches with TMA only
@@ -75,11 +77,6 @@ struct FoldTcParams {
   FoldTcMat mat[KD_MAX_BATCH];
 };
 
-__device__ __forceinline__ void sts128(uint32_t addr, uint4 v) {
-  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
-               : "memory");
-}
-
 // Shared state of a CTA besides the operand ring.
 struct Ctl {
   uint64_t full_a[kMaxA], empty_a[kMaxA], full_b[kMaxB], empty_b[kMaxB], acc_full[2], acc_empty[2];
@@ -87,26 +84,18 @@ struct Ctl {
   int fail;  // a wait expired: the tile's outputs become NaN
 };
 
-// Bounded wait; false once a wait of this CTA has expired (every later one then gives up
-// at once).
-__device__ __forceinline__ bool ctl_wait(Ctl* c, uint64_t* bar, uint32_t parity) {
-  if (mbar_try_wait(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity)) {
-    if (*(volatile int*)&c->fail) return false;
-    if (clock64() - t0 > kWaitCycles) {
-      *(volatile int*)&c->fail = 1;
-      return false;
-    }
-  }
-  return true;
-}
+__device__ __forceinline__ bool ctl_wait(Ctl* c, uint64_t* bar, uint32_t parity) { return tc_wait(bar, parity, &c->fail); }
 
-// resident CTAs per SM; A slots; stages of 64 inputs per B slot: with few rows a slot
-// holds a whole unit, because there the MMA thread's waits and commits cost more than its
-// MMAs; with many rows a slot holds one stage, which keeps more copies in flight
+// Resident CTAs per SM; TMEM columns of a CTA: tc_bufs accumulator buffers of ntc columns,
+// then the A slots; stages of 64 inputs per B slot: with few rows a slot holds a whole unit,
+// because there the MMA thread's waits and commits cost more than its MMAs; with many rows a
+// slot holds one stage, which keeps more copies in flight.
 __host__ __device__ constexpr int tc_ctas(int ntc) { return ntc >= 128 ? 1 : 2; }
-__host__ __device__ constexpr int tc_slots_a(int ntc) { return ntc == 16 || ntc == 128 ? 3 : 2; }
+__host__ __device__ constexpr int tc_cols(int ntc) { return 512 / tc_ctas(ntc); }
+__host__ __device__ constexpr int tc_bufs(int ntc) { return ntc == 256 ? 1 : 2; }
+__host__ __device__ constexpr int tc_slots_a(int ntc) {
+  return (tc_cols(ntc) - tc_bufs(ntc) * ntc) / kACols < kMaxA ? (tc_cols(ntc) - tc_bufs(ntc) * ntc) / kACols : kMaxA;
+}
 __host__ __device__ constexpr int tc_bstages(int ntc) { return ntc >= 128 ? 1 : 2; }
 
 // B tile of rows that TMA cannot read (not 16-byte aligned), by the 256 threads of a decoding
@@ -134,11 +123,11 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
   extern __shared__ uint8_t smem_raw[];
   __shared__ Ctl ctl;
   constexpr int NC = NTC / 4;  // accumulator columns per decoding warp
-  constexpr uint32_t kCols = 2 * NTC < 32 ? 32 : 2 * NTC;
+  constexpr uint32_t kCols = tc_cols(NTC);
+  constexpr int NB = tc_bufs(NTC);
   constexpr int SA = tc_slots_a(NTC);
   constexpr int BH = tc_bstages(NTC);
-  const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;  // the A slots, then the B slots
-  const uint32_t ring_b = ring + SA * kABytes;
+  const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;  // the B slots
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   const int lane = threadIdx.x & 31;
   const int S = p.slots_b;
@@ -219,7 +208,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
           const int k = k0 + (BH == 2 ? i : i >> 1);
           const CUtensorMap* map = k >= ku ? &a.map_xp : &a.map_x;
           const int x = (k >= ku ? k - ku : k) * kUnitK + (BH == 2 ? 0 : (i & 1) * kStageK);
-          uint8_t* dst = smem_raw + (ring_b + s * bbytes - smem_u32(smem_raw));
+          uint8_t* dst = smem_raw + (ring + s * bbytes - smem_u32(smem_raw));
           mbar_arrive_expect_tx(&ctl.full_b[s], bbytes);
 #pragma unroll
           for (int h = 0; h < BH; ++h) tma_load_2d(dst + h * bstage, map, x + h * kStageK, row0, &ctl.full_b[s]);
@@ -234,14 +223,14 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
   } else if (warp == kDecWarps + 1) {
     // ---- MMAs ----
     const uint32_t idesc = tc_idesc(BF, nt);
-    const uint64_t da0 = tc_desc(ring), db0 = tc_desc(ring_b);
+    const uint64_t db0 = tc_desc(ring);
     int s = 0, sa = 0, left = kChunk;  // units left of this accumulation
     uint32_t par = 0, par_a = 0, b = 0, par_acc = 1;
     bool ok = true, fresh = true;
     for (int u = 0; u < L && ok; ++u) {
-      if (u >= 2 * kChunk && fresh) ok = ctl_wait(&ctl, &ctl.acc_empty[b], par_acc);
+      if (u >= NB * kChunk && fresh) ok = ctl_wait(&ctl, &ctl.acc_empty[b], par_acc);
       ok = ok && ctl_wait(&ctl, &ctl.full_a[sa], par_a);
-      const uint64_t da = da0 + (uint64_t)(sa * (kABytes >> 4));
+      const uint32_t ta = tmem + NB * NTC + sa * kACols;
       const uint32_t d = tmem + b * NTC;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -253,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
           const uint64_t db = db0 + (uint64_t)(s * (bbytes >> 4)) + (BH == 2 ? h * (bstage >> 4) : 0u);
 #pragma unroll
           for (int q = 0; q < kStageK / 16; ++q)
-            tc_mma(d, da + h * (kABytes / 2 / 16) + 2 * q, db + 2 * q, idesc, !fresh || h + q != 0);
+            tc_mma_ta(d, ta + 32 * h + 8 * q, db + 2 * q, idesc, !fresh || h + q != 0);
           if (BH == 1 || h == 1) tc_commit(&ctl.empty_b[s]);
           if (h == 1) {
             tc_commit(&ctl.empty_a[sa]);
@@ -273,7 +262,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
       fresh = --left == 0;
       if (fresh) {
         left = kChunk;
-        b ^= 1;
+        if (NB == 2) b ^= 1;
         if (b == 0) par_acc ^= 1;
       }
     }
@@ -284,16 +273,15 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
   if (warp < kDecWarps) {
     // ---- decode, and the fp32 sums ----
     const uint2 cu = centre_bytes<BF>(a.centres_u, c0 + r, live), cv = centre_bytes<BF>(a.centres_v, c0 + r, live);
-    // row r of an A tile, its swizzle in the low bits: chunk c sits at at ^ (c << 4)
-    const uint32_t at = ring + half * (kABytes / 2) + r * 128u + ((r & 7u) << 4);
+    const uint32_t lanes = tmem + ((uint32_t)(warp & 3) << 21);  // this warp's 32 TMEM lanes
 #pragma unroll
     for (int i = 0; i < NC; ++i) acc[i] = 0.f;
     int done = 0;  // chunks added so far
     auto promote = [&]() {
-      const int b = done & 1;
-      ctl_wait(&ctl, &ctl.acc_full[b], (done >> 1) & 1);
+      const int b = NB == 2 ? done & 1 : 0;
+      ctl_wait(&ctl, &ctl.acc_full[b], (NB == 2 ? done >> 1 : done) & 1);
       tc_fence_after();
-      const uint32_t t = tmem + b * NTC + ((uint32_t)(warp & 3) << 21) + (warp >> 2) * NC;
+      const uint32_t t = lanes + b * NTC + (warp >> 2) * NC;
 #pragma unroll
       for (int q = 0; q < NC; q += 16) {
         constexpr int W = NC < 16 ? NC : 16;
@@ -317,23 +305,20 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
       w1 = fetch(u + 4);
       const int s = u % SA;
       if (u >= SA) ctl_wait(&ctl, &ctl.empty_a[s], (u / SA - 1) & 1);
-      // the slot is free: the MMAs up to unit u - SA are complete
-      if ((done + 1) * kChunk <= u - SA + 1) promote();
+      tc_fence_after();  // the MMAs that read the slot are complete
       const bool v = k0 + u >= ku;
       const uint2 c = make_uint2(v ? cv.x : cu.x, v ? cv.y : cu.y);
-      const uint32_t base = at + s * kABytes;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         uint4 e0, e1;
         decode_word(ww[q], c, p.mul, e0, e1);
-        sts128(base ^ ((2 * q) << 4), e0);
-        sts128(base ^ ((2 * q + 1) << 4), e1);
+        tmem_st8(lanes + NB * NTC + s * kACols + 32 * half + 8 * q, e0, e1);
       }
       if constexpr (!TMA) {
         for (int h = 0; h < 2; ++h) {
           const int i = BH == 2 ? u : 2 * u + h, sb = i % S;
           if (i >= S) ctl_wait(&ctl, &ctl.empty_b[sb], (i / S - 1) & 1);
-          fill_rows(ring_b + sb * bbytes + (BH == 2 ? h * bstage : 0u), (v ? a.xp : a.x) + row0 * a.ldx, a.ldx,
+          fill_rows(ring + sb * bbytes + (BH == 2 ? h * bstage : 0u), (v ? a.xp : a.x) + row0 * a.ldx, a.ldx,
                     (int64_t)kUnitK * (v ? k0 + u - ku : k0 + u) + h * kStageK, a.n, nt, p.rows - row0, threadIdx.x & (2 * kTile - 1));
           if (BH == 1 || h == 1) {
             fence_proxy_async_smem();
@@ -342,9 +327,13 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
           }
         }
       }
-      fence_proxy_async_smem();  // the tile's writes before the MMA's reads
+      tmem_wait_st();
+      tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl.full_a[s]);
+      // past the end of an accumulation (with two buffers, when its MMAs are known to be
+      // complete): they need nothing more from this warp
+      if (u >= (done + 1) * kChunk + (NB == 2 ? SA - 1 : 0)) promote();
     }
     const int chunks = (L + kChunk - 1) / kChunk;
     while (done < chunks) promote();
@@ -433,11 +422,11 @@ bool encode_rows(CUtensorMap* map, const void* x, int64_t n, int64_t rows, int64
 template <bool BF, int NTC, bool TMA>
 cudaError_t launch_tc(FoldTcParams& p, int64_t tiles, cudaStream_t s) {
   const int budget = tc_ctas(NTC) == 1 ? 224 * 1024 : 110 * 1024;
-  constexpr int kA = tc_slots_a(NTC) * kABytes;
   const int slot = tc_bstages(NTC) * p.nt * 128;
-  const int left = (budget - kA) / slot;
+  const int left = budget / slot;
   p.slots_b = left < kMaxB ? left : kMaxB;
-  const size_t smem = (size_t)kA + (size_t)p.slots_b * slot + 1024;
+  // at least what the partial tiles of a split take at the end
+  const size_t smem = (size_t)p.slots_b * slot + 1024;
   auto kernel = fold16_tc_kernel<BF, NTC, TMA>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -1,0 +1,459 @@
+// The folded 2-bit layer product of App. C in fp32 (kd_fold.cu states it) on the tensor
+// cores, for two batch rows and more, with nothing rounded to 16 bits.
+//
+//  * An input is the exact sum of three bf16 values, x = x1 + x2 + x3 (truncated to 8
+//    significant bits, the rest, and what that leaves: 24 bits).
+//  * A weight enters as which code it has, not as its centre: with T_q the sum of the inputs
+//    whose code is q, the product of one plane is c0 T0 + c1 T1 + c2 T2 + c3 T3.  The MMAs
+//    multiply the inputs by planes of -1, 0 and 1, which are exact in bf16:
+//        D_in = T2 - T1, D_out = T3 - T0, and where a channel of the tile has centres that are
+//        not symmetric about 0 (after k-means refinement), E_in = T1 + T2, E_out = T0 + T3.
+//    The centres stay fp32 and multiply the sums.
+// Products are exact, and so are most additions inside the tensor core (an 8-bit value and a
+// sum of a few hundred of them); every kChunk stages the sums move to fp32 registers.
+//
+// Mapping.  tcgen05.mma with M = 128 output channels, N = 3 values per batch row (16 rows per
+// block), K = the inputs in stages of 64.  A cluster of two CTAs owns a tile of 128 channels:
+// CTA 0 the u plane with x, CTA 1 the v plane with xp; their sums are added at the end over
+// distributed shared memory.  In a CTA
+//  * two groups of four warps decode, every other stage each: a thread turns the four code
+//    words of its channel into its TMEM lane of either plane (the MMA takes A from TMEM:
+//    through shared memory, the planes' writes and reads filled its bandwidth and 16 rows of
+//    the 7B layer took 190 us);
+//  * two groups of two warps split the inputs into the B tile in shared memory, every other
+//    stage each, their loads two own stages ahead (the inputs come from L2);
+//  * one thread issues the MMAs;
+//  * the decoding warps also move finished sums from TMEM to registers.
+// With centres that are not symmetric the K loop runs twice, over the D and then the E planes.
+// TMEM (256 of 512 columns, two CTAs per SM): the sums of two planes, and one slot of A for
+// each decoding group; while one CTA waits for its slot or its sums, the other decodes.
+//
+// Rows and channels with an infinity, a NaN or a magnitude of 2^101 and more (in the inputs,
+// in the centres) cannot be split or summed without their weights: their outputs are summed
+// again by plain fp32 FMAs.
+//
+// Measured (7B layer, L2 cold): 116 us at 2 rows, 126 at 16, 429 at 64; the table-lookup
+// kernel took 121 us per two rows (970 at 16).  Error against 64 bits at 16 rows, 2-norm:
+// 6e-8 to 8e-8, against 1.6e-7 to 2.2e-7 before (1.0e-7 with centres that are not
+// symmetric).  The ALU pipe is 68 % busy with the decode and the split of the inputs.
+#include <cuda_runtime.h>
+
+#include "kashin.h"
+#include "kd_dec16.cuh"
+#include "kd_fold_tc.h"
+#include "kd_tc.cuh"
+
+namespace kd {
+namespace {
+
+constexpr int kTile = 128;     // output channels per CTA (the MMA's M, the TMEM lanes)
+constexpr int kRows = 16;      // batch rows per block
+constexpr int kStageK = 64;    // inputs per stage
+constexpr int kChunk = 32;     // stages per TMEM accumulation
+constexpr int kDecWarps = 8;   // decoding warps: two groups of four
+constexpr int kSplitWarps = 4;  // two groups of two
+constexpr int kThreads = 32 * (kDecWarps + kSplitWarps + 1);
+constexpr int kSlotsA = 2, kSlotsB = 4;    // A in TMEM, B in shared memory
+constexpr int kBBytes = 3 * kRows * 128;
+constexpr int kSmem = kSlotsB * kBBytes + 1024;
+constexpr uint32_t kCols = 256;            // TMEM: sums of plane p at 64 p, A slot s at 128 + 64 s (32 per plane)
+constexpr uint32_t kBig = 0x72000000u;     // bits of 2^101
+
+struct FoldTcMat {
+  const uint32_t* codes[2];
+  const float* centres[2];
+  const float* x[2];
+  float* y;
+  int64_t n, m, words, ldx, ldy;
+  int vec_codes;  // code rows 16-byte aligned
+  int vec_x;      // input rows of whole 16-byte blocks
+};
+
+struct FoldTcParams {
+  uint32_t tile0[KD_MAX_BATCH];  // first channel tile of each matrix
+  int count;
+  int rows;        // batch rows of the call
+  int row_blocks;  // blocks of kRows rows
+  DecodeMul mul;
+  FoldTcMat mat[KD_MAX_BATCH];
+};
+
+struct Ctl {
+  uint64_t full_a[kSlotsA], empty_a[kSlotsA], full_b[kSlotsB], empty_b[kSlotsB], acc_full, acc_empty;
+  uint32_t tmem;
+  int fail;   // a wait expired: the tile's outputs become NaN
+  int plain;  // batch rows (bits) to be summed by plain FMAs
+};
+
+__device__ __forceinline__ bool ctl_wait(Ctl& c, uint64_t* bar, uint32_t parity) { return tc_wait(bar, parity, &c.fail); }
+
+// code -> bf16 as (low bytes, high bytes) of codes 0..3
+__device__ __forceinline__ uint2 plane_bytes(int p) {
+  return p == 0   ? make_uint2(0x00808000u, 0x003FBF00u)   // D_in:  0 -1  1  0
+         : p == 1 ? make_uint2(0x80000080u, 0x3F0000BFu)   // D_out: -1 0  0  1
+         : p == 2 ? make_uint2(0x00808000u, 0x003F3F00u)   // E_in:  0  1  1  0
+                  : make_uint2(0x80000080u, 0x3F00003Fu);  // E_out: 1  0  0  1
+}
+
+__global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_constant__ FoldTcParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ Ctl ctl;
+  const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;  // the B slots
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+  const int lane = threadIdx.x & 31;
+
+  const uint32_t pl = cluster_rank();  // 0: u plane and x, 1: v plane and xp
+  const uint32_t id = blockIdx.x / 2;
+  const uint32_t tile = id / (uint32_t)p.row_blocks;
+  const int row0 = (int)(id - tile * p.row_blocks) * kRows;
+  int mi = 0;
+  while (mi + 1 < p.count && tile >= p.tile0[mi + 1]) ++mi;
+  const FoldTcMat& a = p.mat[mi];
+  const int64_t c0 = (int64_t)(tile - p.tile0[mi]) * kTile;
+  const int rows = p.rows - row0 < kRows ? p.rows - row0 : kRows;
+  const int nt = (3 * rows + 15) / 16 * 16;
+  const int L = (int)((a.n + kStageK - 1) / kStageK);  // stages
+
+  // decoding threads: channel r of the tile, its centres, its first code words
+  const int grp = warp >> 2;
+  const int r = threadIdx.x & (kTile - 1);
+  const bool live = warp < kDecWarps && c0 + r < a.m;
+  const uint32_t* code_row = a.codes[pl] + (live ? c0 + r : 0) * a.words;
+  const int words = live ? (int)a.words : 0;
+  const bool vec = a.vec_codes;
+  auto fetch = [&](int st) -> uint4 {  // the words of stage st (of either pass), zero past the row and m
+    const int s = st < L ? st : st - L;
+    const int w0 = 4 * s;
+    const int left = words - w0;
+    uint4 w = make_uint4(0u, 0u, 0u, 0u);
+    if (vec) {
+      if (left > 0) w = __ldg(reinterpret_cast<const uint4*>(code_row + w0));
+    } else {
+      if (left > 0) w.x = __ldg(code_row + w0);
+      if (left > 1) w.y = __ldg(code_row + w0 + 1);
+      if (left > 2) w.z = __ldg(code_row + w0 + 2);
+      if (left > 3) w.w = __ldg(code_row + w0 + 3);
+    }
+    return w;
+  };
+  uint4 w0 = fetch(grp), w1 = fetch(grp + 2), w2 = fetch(grp + 4);
+  float4 cen = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (live) cen = __ldg(reinterpret_cast<const float4*>(a.centres[pl]) + c0 + r);
+  auto mag = [](float f) { return __float_as_uint(f) & 0x7FFFFFFFu; };
+  const bool plain_channel = max(max(mag(cen.x), mag(cen.y)), max(mag(cen.z), mag(cen.w))) >= kBig;
+
+  if (warp == kDecWarps + kSplitWarps) {
+    if (lane < kSlotsA) {
+      mbar_init(&ctl.full_a[lane], 4);  // the warps of a decoding group
+      mbar_init(&ctl.empty_a[lane], 1);
+    }
+    if (lane < kSlotsB) {
+      mbar_init(&ctl.full_b[lane], kSplitWarps / 2);
+      mbar_init(&ctl.empty_b[lane], 1);
+    }
+    if (lane == 0) {
+      mbar_init(&ctl.acc_full, 1);
+      mbar_init(&ctl.acc_empty, kDecWarps);
+      ctl.fail = 0;
+      ctl.plain = 0;
+    }
+    mbar_init_fence();
+    tmem_alloc(&ctl.tmem, kCols);
+  }
+  tc_fence_before();
+  // centres symmetric about 0 in the whole tile: two planes suffice
+  const int reps = __syncthreads_or(!(cen.x == -cen.w && cen.y == -cen.z)) ? 2 : 1;
+  tc_fence_after();
+  const uint32_t tmem = ctl.tmem;
+  const int V = L * reps;  // stages of all passes
+  // accumulations of one pass: kChunk stages each but the last
+  const int chunks = (L + kChunk - 1) / kChunk;
+
+  float acc[8];  // batch rows 8 grp .. + 7 of this channel
+#pragma unroll
+  for (int k = 0; k < 8; ++k) acc[k] = 0.f;
+  if (warp == kDecWarps + kSplitWarps) {
+    // ---- MMAs ----
+    const uint32_t idesc = tc_idesc(true, nt);
+    const uint64_t db0 = tc_desc(ring);
+    int in_pass = 0, in_chunk = 0, chunk = 0;
+    bool ok = true;
+    for (int i = 0; i < V && ok; ++i) {
+      if (in_chunk == 0 && chunk > 0) ok = ctl_wait(ctl, &ctl.acc_empty, (chunk - 1) & 1);
+      const int sa = i % kSlotsA, sb = i % kSlotsB;
+      ok = ok && ctl_wait(ctl, &ctl.full_b[sb], (i / kSlotsB) & 1);
+      ok = ok && ctl_wait(ctl, &ctl.full_a[sa], (i / kSlotsA) & 1);
+      tc_fence_after();
+      const bool end = in_chunk == kChunk - 1 || in_pass == L - 1;
+      if (ok && elect_one()) {
+        const uint32_t ta = tmem + 128 + 64 * sa;
+        const uint64_t db = db0 + (uint64_t)(sb * (kBBytes >> 4));
+#pragma unroll
+        for (int pn = 0; pn < 2; ++pn)
+#pragma unroll
+          for (int q = 0; q < kStageK / 16; ++q)
+            tc_mma_ta(tmem + pn * 64, ta + pn * 32 + 8 * q, db + 2 * q, idesc, in_chunk != 0 || q != 0);
+        tc_commit(&ctl.empty_a[sa]);
+        tc_commit(&ctl.empty_b[sb]);
+        if (end) tc_commit(&ctl.acc_full);
+      }
+      __syncwarp();
+      ++in_chunk;
+      ++in_pass;
+      if (end) {
+        in_chunk = 0;
+        ++chunk;
+        if (in_pass == L) in_pass = 0;
+      }
+    }
+  } else if (warp >= kDecWarps) {
+    // ---- B tiles: thread (row t / 8 + 8 h, inputs 8 (t % 8) .. + 7), h = 0, 1 ----
+    const int sg = (warp - kDecWarps) >> 1;
+    const int t = threadIdx.x & 63;
+    const int seg = t & 7, br0 = t >> 3;
+    const float* src = a.x[pl] + (int64_t)(row0 + br0) * a.ldx + 8 * seg;
+    const bool vec_x = a.vec_x;
+    uint32_t big[2] = {0u, 0u};
+    auto load = [&](int st, float (&v)[2][8]) {
+      const int i0 = kStageK * (st < L ? st : st - L);
+      const int left = (int)(a.n - i0 - 8 * seg);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float* q = src + 8 * h * a.ldx + i0;
+        const bool in = st < V && br0 + 8 * h < rows;
+        if (vec_x) {
+          float4 f0 = make_float4(0.f, 0.f, 0.f, 0.f), f1 = f0;
+          if (in && left >= 4) f0 = __ldg(reinterpret_cast<const float4*>(q));
+          if (in && left >= 8) f1 = __ldg(reinterpret_cast<const float4*>(q) + 1);
+          v[h][0] = f0.x; v[h][1] = f0.y; v[h][2] = f0.z; v[h][3] = f0.w;
+          v[h][4] = f1.x; v[h][5] = f1.y; v[h][6] = f1.z; v[h][7] = f1.w;
+        } else {
+#pragma unroll
+          for (int e = 0; e < 8; ++e) v[h][e] = in && e < left ? __ldg(q + e) : 0.f;
+        }
+      }
+    };
+    auto put = [&](int s, const float (&v)[2][8]) {
+      const int sb = s % kSlotsB;
+      if (s >= kSlotsB) ctl_wait(ctl, &ctl.empty_b[sb], (s / kSlotsB - 1) & 1);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int br = br0 + 8 * h;
+        if (br < rows) {
+          uint32_t pk[3][4];
+#pragma unroll
+          for (int e = 0; e < 8; e += 2) {
+            // K order inside 8 inputs as the decoded codes': 0, 4, 1, 5, 2, 6, 3, 7
+            uint32_t b1[2], b2[2], b3[2];
+#pragma unroll
+            for (int o = 0; o < 2; ++o) {
+              const float x = v[h][e / 2 + 4 * o];
+              const uint32_t bits = __float_as_uint(x);
+              big[h] = max(big[h], bits & 0x7FFFFFFFu);
+              b1[o] = bits & 0xFFFF0000u;
+              const float rest = __fsub_rn(x, __uint_as_float(b1[o]));
+              b2[o] = __float_as_uint(rest) & 0xFFFF0000u;
+              b3[o] = __float_as_uint(__fsub_rn(rest, __uint_as_float(b2[o])));
+            }
+            pk[0][e / 2] = prmt(b1[0], b1[1], 0x7632u);
+            pk[1][e / 2] = prmt(b2[0], b2[1], 0x7632u);
+            pk[2][e / 2] = prmt(b3[0], b3[1], 0x7632u);
+          }
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const uint32_t row = 3 * br + q;
+            sts128(ring + sb * kBBytes + row * 128 + ((seg ^ (row & 7)) << 4),
+                   make_uint4(pk[q][0], pk[q][1], pk[q][2], pk[q][3]));
+          }
+        }
+      }
+      fence_proxy_async_smem();  // the tile's writes before the MMA's reads
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.full_b[sb]);
+    };
+    float va[2][8], vb[2][8];
+    load(sg, va);
+    load(sg + 2, vb);
+#pragma unroll 1
+    for (int s = sg; s < V; s += 4) {
+      put(s, va);
+      load(s + 4, va);
+      if (s + 2 < V) put(s + 2, vb);
+      load(s + 6, vb);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (big[h] >= kBig) atomicOr(&ctl.plain, 1 << (br0 + 8 * h));
+  } else {
+    // ---- decode, and the fp32 sums ----
+    const uint32_t lanes = tmem + ((uint32_t)(warp & 3) << 21);  // this warp's 32 TMEM lanes
+    int done = 0, done_stage = 0;  // chunks added so far, the stage that ends the next one
+    auto next_end = [&]() {
+      const int pass = done / chunks, c = done - pass * chunks;
+      done_stage = pass * L + (c + 1 < chunks ? (c + 1) * kChunk : L);
+    };
+    next_end();
+    auto promote = [&]() {
+      ctl_wait(ctl, &ctl.acc_full, done & 1);
+      tc_fence_after();
+      // factors of the inner and the outer plane: c2, c3 where the centres are symmetric,
+      // else half of c2 - c1, c3 - c0 for D and of c2 + c1, c3 + c0 for E
+      float fi = cen.z, fo = cen.w;
+      if (reps == 2) {
+        const bool e = done >= chunks;
+        fi = __fmul_rn(0.5f, e ? __fadd_rn(cen.z, cen.y) : __fsub_rn(cen.z, cen.y));
+        fo = __fmul_rn(0.5f, e ? __fadd_rn(cen.w, cen.x) : __fsub_rn(cen.w, cen.x));
+      }
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {  // four batch rows, twelve columns
+        if (8 * grp + 4 * half < rows) {
+          float d[2][12];
+#pragma unroll
+          for (int pn = 0; pn < 2; ++pn)
+#pragma unroll
+            for (int q = 0; q < 12; q += 4) tmem_ld4(&d[pn][q], lanes + pn * 64 + 24 * grp + 12 * half + q);
+          tmem_wait_ld();
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            // the three parts of the inputs, the smallest first
+            const float in = __fadd_rn(__fadd_rn(d[0][3 * k + 2], d[0][3 * k + 1]), d[0][3 * k]);
+            const float out = __fadd_rn(__fadd_rn(d[1][3 * k + 2], d[1][3 * k + 1]), d[1][3 * k]);
+            acc[4 * half + k] = __fadd_rn(acc[4 * half + k], __fmaf_rn(fo, out, __fmul_rn(fi, in)));
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.acc_empty);
+      ++done;
+      next_end();
+    };
+    // own stages grp, grp + 2, ..., their code words loaded three own stages ahead
+#pragma unroll 1
+    for (int i = grp; i < V; i += 2) {
+      const uint32_t ww[4] = {w0.x, w0.y, w0.z, w0.w};
+      w0 = w1;
+      w1 = w2;
+      w2 = fetch(i + 6);
+      const bool e = i >= L;
+      const uint2 b0 = plane_bytes(e ? 2 : 0), b1 = plane_bytes(e ? 3 : 1);
+      if (i >= kSlotsA) ctl_wait(ctl, &ctl.empty_a[grp], (i / kSlotsA - 1) & 1);
+      tc_fence_after();  // the MMAs that read the slot are complete
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint32_t sel[8];
+        uint4 lo, hi;
+        decode_selectors_by4(ww[q], p.mul, sel);
+        decode_pick(sel, b0, lo, hi);
+        tmem_st8(lanes + 128 + 64 * grp + 8 * q, lo, hi);
+        decode_pick(sel, b1, lo, hi);
+        tmem_st8(lanes + 160 + 64 * grp + 8 * q, lo, hi);
+      }
+      tmem_wait_st();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&ctl.full_a[grp]);
+      // past the end of an accumulation: its MMAs need nothing more from this warp.  All that
+      // ended: a pass may end in an accumulation of one stage, and then the other group's
+      // next slot waits for this one's sums
+      while (done < chunks * reps && i >= done_stage) promote();
+    }
+    while (done < chunks * reps) promote();
+  }
+
+  __syncthreads();  // the MMAs have completed (their sums were waited for): shared memory is free
+  const int plain = *(volatile int*)&ctl.plain;
+  const float bad = *(volatile int*)&ctl.fail ? __int_as_float(0x7FC00000) : 0.f;
+  if (warp < kDecWarps) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int c = 8 * grp + k;
+      float v = acc[k];
+      if (c < rows && (plain_channel || ((plain >> c) & 1))) {
+        v = 0.f;
+        const float* q = a.x[pl] + (int64_t)(row0 + c) * a.ldx;
+        const float cc[4] = {cen.x, cen.y, cen.z, cen.w};
+        for (int64_t i = 0; live && i < a.n; ++i) {
+          const uint32_t code = (__ldg(code_row + (i >> 4)) >> (2 * (int)(i & 15))) & 3u;
+          const float ce = (code & 2u) ? ((code & 1u) ? cc[3] : cc[2]) : ((code & 1u) ? cc[1] : cc[0]);
+          v = __fmaf_rn(ce, __ldg(q + i), v);
+        }
+      }
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + r) * 4), "f"(__fadd_rn(v, bad)) : "memory");
+    }
+  }
+  cluster_sync_all();
+  // CTA 0 writes the even batch rows, CTA 1 the odd ones: u plane first
+  if (live) {
+    for (int c = 2 * grp + (int)pl; c < rows; c += 4) {
+      const uint32_t at = ring + (c * kTile + r) * 4;
+      a.y[(int64_t)(row0 + c) * a.ldy + c0 + r] = __fadd_rn(ld_dsmem(at, 0), ld_dsmem(at, 1));
+    }
+  }
+  cluster_sync_all();  // the peer's reads of this CTA's shared memory are done
+  if (warp == kDecWarps + kSplitWarps) tmem_dealloc(tmem, kCols);
+}
+
+bool aligned_to(const void* ptr, size_t a) { return reinterpret_cast<uintptr_t>(ptr) % a == 0; }
+
+}  // namespace
+
+kd_status fold_tc_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStream_t s) {
+  // channel tiles numbered longest vectors first, so that the long ones of a layer are not
+  // the last ones started
+  int order[KD_MAX_BATCH];
+  for (int i = 0; i < count; ++i) order[i] = i;
+  for (int i = 1; i < count; ++i)
+    for (int k = i; k > 0 && mats[order[k]].n > mats[order[k - 1]].n; --k) {
+      const int tmp = order[k];
+      order[k] = order[k - 1];
+      order[k - 1] = tmp;
+    }
+  cudaError_t e = cudaFuncSetAttribute(fold_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e != cudaSuccess) return KD_ERR_CUDA;
+  constexpr int64_t kMaxRows = 1 << 16;  // batch rows per launch
+  for (int64_t b0 = 0; b0 < batch; b0 += kMaxRows) {
+    FoldTcParams p;
+    p.rows = (int)(batch - b0 < kMaxRows ? batch - b0 : kMaxRows);
+    p.row_blocks = (p.rows + kRows - 1) / kRows;
+    p.count = 0;
+    int64_t tiles = 0;
+    for (int i = 0; i < count; ++i) {
+      const kd_fold_mat& a = mats[order[i]];
+      if (a.m == 0) continue;
+      p.tile0[p.count] = (uint32_t)tiles;
+      FoldTcMat& f = p.mat[p.count++];
+      f.codes[0] = a.codes_u;
+      f.codes[1] = a.codes_v;
+      f.centres[0] = a.centres_u;
+      f.centres[1] = a.centres_v;
+      f.x[0] = a.x + b0 * a.ldx;
+      f.x[1] = a.xp + b0 * a.ldx;
+      f.y = a.y + b0 * a.ldy;
+      f.n = a.n;
+      f.m = a.m;
+      f.words = (a.n + 15) / 16;
+      f.ldx = a.ldx;
+      f.ldy = a.ldy;
+      f.vec_codes = aligned_to(a.codes_u, 16) && aligned_to(a.codes_v, 16) && f.words % 4 == 0;
+      f.vec_x = aligned_to(f.x[0], 16) && aligned_to(f.x[1], 16) && a.ldx % 4 == 0 && a.n % 4 == 0;
+      tiles += (a.m + kTile - 1) / kTile;
+    }
+    if (tiles == 0) return KD_OK;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(tiles * p.row_blocks * 2));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, fold_tc_kernel, p) != cudaSuccess) return KD_ERR_CUDA;
+  }
+  return KD_OK;
+}
+
+}  // namespace kd

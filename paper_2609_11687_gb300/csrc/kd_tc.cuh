@@ -57,6 +57,23 @@ __device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b, uint3
       : "memory");
 }
 
+// the same with A in TMEM: lane = row, each 32-bit column two consecutive K entries
+__device__ __forceinline__ void tc_mma_ta(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, bool accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"((uint32_t)accumulate)
+      : "memory");
+}
+
+// eight 32-bit columns of this warp's 32 TMEM lanes; complete after tmem_wait_st
+__device__ __forceinline__ void tmem_st8(uint32_t addr, uint4 lo, uint4 hi) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr), "r"(lo.x),
+               "r"(lo.y), "r"(lo.z), "r"(lo.w), "r"(hi.x), "r"(hi.y), "r"(hi.z), "r"(hi.w)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // arrives on bar once every tcgen05.mma this thread issued before has completed
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
@@ -76,6 +93,14 @@ __device__ __forceinline__ void tmem_ld8(float* v, uint32_t addr) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_ld4(float* v, uint32_t addr) {  // four columns
+  uint32_t r[4];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) v[i] = __uint_as_float(r[i]);
+}
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -90,6 +115,34 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
           smem_u32(dst)),
       "l"(map), "r"(c0), "r"(c1), "r"(smem_u32(bar))
       : "memory");
+}
+
+// Bounded wait for the phase of `bar` with this parity: false, with *fail set, once a wait of
+// this CTA has taken longer than kWaitCycles (every later one then gives up at once).  The
+// suspend-time hint (10 ms) lets the hardware park the thread: polling took a tenth of the
+// issue slots from the decoding warps.
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* fail) {
+  auto parked = [&]() {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(10000000u)
+        : "memory");
+    return done != 0;
+  };
+  if (parked()) return true;
+  const long long t0 = clock64();
+  while (!parked()) {
+    if (*(volatile int*)fail) return false;
+    if (clock64() - t0 > kWaitCycles) {
+      *(volatile int*)fail = 1;
+      return false;
+    }
+  }
+  return true;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {
