@@ -54,27 +54,6 @@ struct WsLayout {
   size_t status, eps, tw, uslots, total;
 };
 
-// sign bits of several matrices: set i at eps + i * words (batched launches)
-struct SeedList {
-  int count, words;
-  int64_t n;
-  uint64_t seed[kMaxBatch];
-};
-
-__global__ void eps_batch_kernel(uint32_t* eps, SeedList sl) {
-  const int total = sl.count * sl.words;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < total; g += gridDim.x * blockDim.x) {
-    const int i = g / sl.words, wd = g - i * sl.words;
-    uint32_t bits = 0;
-    for (int bb = 0; bb < 32; ++bb) {
-      const int64_t j = (int64_t)wd * 32 + bb;
-      if (j >= sl.n) break;
-      bits |= (uint32_t)(splitmix64_mix(sl.seed[i] + (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull) >> 63) << bb;
-    }
-    eps[g] = bits;
-  }
-}
-
 int sm_count() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -106,28 +85,23 @@ bool layout_of(const PlanOps* ops, WsLayout* L, int nsets = 1) {
   return true;
 }
 
-kd_status setup(const PlanOps* ops, const WsLayout& L, void* ws, uint64_t seed, cudaStream_t s) {
-  char* b = static_cast<char*>(ws);
-  cudaError_t e = ops->setup(reinterpret_cast<float2*>(b + L.tw), reinterpret_cast<uint32_t*>(b + L.eps),
-                             reinterpret_cast<uint32_t*>(b + L.status), seed, ops->n, s);
-  return e == cudaSuccess ? KD_OK : KD_ERR_CUDA;
-}
-
-// Tables of a batched call: twiddles, status and sign set 0 from the first seed, then
-// sign sets 1 .. count-1 (set i at eps + i * ceil(n / 32)).
+// Tables of a call: twiddles, the cleared status word and the sign sets of its matrices
+// (set i at eps + i * ceil(n / 32)).
 kd_status setup_batch(const PlanOps* ops, const WsLayout& L, void* ws, const uint64_t* seeds, int count, int64_t n,
                       cudaStream_t s) {
-  kd_status st = setup(ops, L, ws, seeds[0], s);
-  if (st != KD_OK || count == 1) return st;
   SeedList sl;
   sl.count = count;
   sl.words = (int)((n + 31) / 32);
-  sl.n = n;
+  sl.n = (int)n;
   for (int i = 0; i < count; ++i) sl.seed[i] = seeds[i];
-  const int total = count * sl.words;
-  eps_batch_kernel<<<(total + 255) / 256, 256, 0, s>>>(reinterpret_cast<uint32_t*>(static_cast<char*>(ws) + L.eps),
-                                                       sl);
-  return cudaGetLastError() == cudaSuccess ? KD_OK : KD_ERR_CUDA;
+  char* b = static_cast<char*>(ws);
+  const cudaError_t e = ops->setup(reinterpret_cast<float2*>(b + L.tw), reinterpret_cast<uint32_t*>(b + L.eps),
+                                   reinterpret_cast<uint32_t*>(b + L.status), sl, n, s);
+  return e == cudaSuccess ? KD_OK : KD_ERR_CUDA;
+}
+
+kd_status setup(const PlanOps* ops, const WsLayout& L, void* ws, uint64_t seed, cudaStream_t s) {
+  return setup_batch(ops, L, ws, &seed, 1, ops->n, s);
 }
 
 int grid_for(int64_t npairs, int q, int ctas_max) {

@@ -123,22 +123,26 @@ __global__ void __launch_bounds__(kGenThreads, 2) gen_reconstruct_kernel(RecPara
   }
 }
 
-// Tables of one call: pass twiddles, exp(i pi k/n), frequency slots, sign bits
-// (SplitMix64, as the per-length set-up) and the cleared status word.
-__global__ void gen_setup_kernel(float2* tab, uint32_t* eps, uint32_t* status, uint64_t seed,
+// Tables of one call: pass twiddles, exp(i pi k/n), group bases, addresses by position and by
+// frequency, sign bits (setup_signs) and the cleared status word.  One entry per thread, the
+// kinds one after another, each from a block of its own.
+__host__ __device__ inline int gen_setup_blocks(const GenPlan& g, int (&first)[6]) {
+  int bases = 0;
+  for (int i = 0; i < g.np - g.fused; ++i) bases += g.n / g.R[i];
+  const int freqs = g.fused ? g.n / g.R[g.np - 1] : g.n;
+  const int len[5] = {g.woff, g.n / 2 + 1, bases, g.n, freqs};
+  first[0] = 0;
+  for (int i = 0; i < 5; ++i) first[i + 1] = first[i] + (len[i] + kSetupThreads - 1) / kSetupThreads;
+  return first[5];
+}
+
+__global__ void gen_setup_kernel(float2* tab, uint32_t* eps, uint32_t* status, const __grid_constant__ SeedList sl,
                                  const __grid_constant__ GenPlan g) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int stride = gridDim.x * blockDim.x;
+  int first[6];
+  gen_setup_blocks(g, first);
+  const int blk = blockIdx.x;
   const int n = g.n;
-  if (tid == 0) *status = 0u;
-  for (int e = tid; e < g.woff; e += stride) {
-    int i = 0;
-    while (i + 1 < g.np - 1 && e >= g.tw[i + 1]) ++i;
-    const int r = e - g.tw[i];
-    const int sp = r % g.S[i], j = r / g.S[i];
-    tab[e] = root_w((long long)sp * j, g.B[i]);
-  }
-  for (int k = tid; 2 * k <= n; k += stride) tab[g.woff + k] = expi_pi(k, n);
+  if (blk == 0 && threadIdx.x == 0) *status = 0u;
   auto address = [&](int s) {  // of slot s
     int at = 0;
     for (int i = 0; i < g.np; ++i) {
@@ -148,33 +152,40 @@ __global__ void gen_setup_kernel(float2* tab, uint32_t* eps, uint32_t* status, u
     }
     return at;
   };
-  for (int i = 0; i < g.np - g.fused; ++i) {
-    uint32_t* base = reinterpret_cast<uint32_t*>(tab) + g.base[i];
-    for (int k = tid; k < n / g.R[i]; k += stride) {
-      const int blk = k / g.S[i], sp = k - blk * g.S[i];
-      base[k] = (uint32_t)address(blk * g.B[i] + sp) | (uint32_t)sp << 16;
-    }
-  }
   uint16_t* at16 = reinterpret_cast<uint16_t*>(tab);
-  for (int s = tid; s < n; s += stride) at16[g.addroff + s] = (uint16_t)address(s);
-  const int groups = g.fused ? n / g.R[g.np - 1] : n;
-  for (int k = tid; k < groups; k += stride) {
+  if (blk < first[1]) {
+    const int e = blk * kSetupThreads + threadIdx.x;
+    if (e >= g.woff) return;
+    int i = 0;
+    while (i + 1 < g.np - 1 && e >= g.tw[i + 1]) ++i;
+    const int r = e - g.tw[i];
+    const int j = r / g.S[i], sp = r - j * g.S[i];
+    tab[e] = root_w((long long)sp * j, g.B[i]);
+  } else if (blk < first[2]) {
+    const int k = (blk - first[1]) * kSetupThreads + threadIdx.x;
+    if (2 * k <= n) tab[g.woff + k] = expi_pi(k, n);
+  } else if (blk < first[3]) {
+    int k = (blk - first[2]) * kSetupThreads + threadIdx.x;
+    int i = 0;
+    while (i < g.np - g.fused && k >= n / g.R[i]) k -= n / g.R[i++];
+    if (i == g.np - g.fused) return;
+    const int bk = k / g.S[i], sp = k - bk * g.S[i];
+    reinterpret_cast<uint32_t*>(tab)[g.base[i] + k] = (uint32_t)address(bk * g.B[i] + sp) | (uint32_t)sp << 16;
+  } else if (blk < first[4]) {
+    const int s = (blk - first[3]) * kSetupThreads + threadIdx.x;
+    if (s < n) at16[g.addroff + s] = (uint16_t)address(s);
+  } else if (blk < first[5]) {
+    const int k = (blk - first[4]) * kSetupThreads + threadIdx.x;
+    if (k >= (g.fused ? n / g.R[g.np - 1] : n)) return;
     int x = k, s = 0;
     for (int i = 0; i < g.np - g.fused; ++i) {
-      s += (x % g.R[i]) * g.S[i];
-      x /= g.R[i];
+      const int q = x / g.R[i];
+      s += (x - q * g.R[i]) * g.S[i];
+      x = q;
     }
     at16[g.freqoff + k] = (uint16_t)address(s);
-  }
-  const int words = (n + 31) / 32;
-  for (int wd = tid; wd < words; wd += stride) {
-    uint32_t bits = 0;
-    for (int bb = 0; bb < 32; ++bb) {
-      const int j = wd * 32 + bb;
-      if (j >= n) break;
-      bits |= (uint32_t)(splitmix64_mix(seed + (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull) >> 63) << bb;
-    }
-    eps[wd] = bits;
+  } else {
+    setup_signs(eps, sl, first[5]);
   }
 }
 
@@ -250,12 +261,12 @@ cudaError_t gen_reconstruct(const RecParams& p, const RecBatch* rb, int grid, cu
   return cudaGetLastError();
 }
 
-cudaError_t gen_setup(float2* tab, uint32_t* eps, uint32_t* status, uint64_t seed, int64_t n, cudaStream_t s) {
+cudaError_t gen_setup(float2* tab, uint32_t* eps, uint32_t* status, const SeedList& sl, int64_t n, cudaStream_t s) {
   GenPlan g;
   if (!gen_plan(n, &g)) return cudaErrorInvalidValue;
-  const int work = g.twn > n ? g.twn : (int)n;
-  const int blocks = (work + 255) / 256;
-  gen_setup_kernel<<<blocks, 256, 0, s>>>(tab, eps, status, seed, g);
+  int first[6];
+  const int blocks = gen_setup_blocks(g, first) + sl.count * sl.words * 32 / kSetupThreads;
+  gen_setup_kernel<<<blocks, kSetupThreads, 0, s>>>(tab, eps, status, sl, g);
   return cudaGetLastError();
 }
 

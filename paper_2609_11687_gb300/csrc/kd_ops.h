@@ -14,6 +14,14 @@ struct ApplyBatch;
 struct RecParams;
 struct RecBatch;
 
+// Sign sets of one call: matrix i's at eps + i * words (words = ceil(n / 32))
+constexpr int kMaxSeeds = 32;
+struct SeedList {
+  int count, words;
+  int n;
+  uint64_t seed[kMaxSeeds];
+};
+
 struct PlanOps {
   int n;
   int threads;      // threads per CTA
@@ -31,7 +39,7 @@ struct PlanOps {
   // rb: the matrices of a batched launch, or nullptr for RecParams' single matrix
   cudaError_t (*reconstruct)(const RecParams&, const RecBatch* rb, int grid, cudaStream_t);
   // tables for one call of vector length n: twiddles (float2[twn]), sign bits, cleared status word
-  cudaError_t (*setup)(float2* twt, uint32_t* eps, uint32_t* status, uint64_t seed, int64_t n, cudaStream_t);
+  cudaError_t (*setup)(float2* twt, uint32_t* eps, uint32_t* status, const SeedList& seeds, int64_t n, cudaStream_t);
 };
 
 // Argument checks of kd_decompose, in its order and with its status codes (a kd_status

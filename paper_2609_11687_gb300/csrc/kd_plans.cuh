@@ -27,6 +27,13 @@ using Plan11008 = Plan<11008, 256, 1, USMEM, 1, 43, 16, 16>;
 using Plan14336 = Plan<14336, 512, 1, UGMEM, 1, 28, 16, 32>;
 using Plan16384 = Plan<16384, 512, 1, UGMEM, 1, 32, 32, 16>;
 
+// without u the n = 11008 twiddle table (90 KB) fits in shared memory
+template <>
+struct LightPlan<Plan11008> {
+  using type = Plan<11008, 256, 1, UREG, 1, 43, 16, 16>;
+};
+static_assert(LightPlan<Plan11008>::type::TW_SMEM, "the table is staged");
+
 // packed constant roots (2.5 % faster at n = 4096; at n = 11008 the constant pairs
 // cost spills and 9 %)
 template <>

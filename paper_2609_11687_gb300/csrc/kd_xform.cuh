@@ -29,6 +29,7 @@
 #include <type_traits>
 
 #include "kd_math.cuh"
+#include "kd_ops.h"
 
 namespace kd {
 
@@ -281,6 +282,14 @@ struct Xform {
   static constexpr bool WLU = NP == 3 && !PL::PAIRED && (E % 2 == 1) && PL::R(1) == 16 && PL::RL == 16 &&
                               PL::S(1) == 16 && T == 256;
   static constexpr int NU = (E + 1) / 2;  // units
+  // M's per-thread roots, after the twiddles in the table (derived by the set-up kernel: a
+  // double-precision sincospi per thread took 3 us of every launch, three of them 10 us at
+  // n = 11008): entry c is exp(i pi c / N) by last-pass group (by exp(i pi E c / N) for slot-
+  // order plans)
+  static constexpr int CWN = WLU ? N / 16 : T;
+  __device__ static __forceinline__ float2 cw_entry(int c) {
+    return expi_pi((PL::PAIRED || WLU) ? (long long)c : (long long)E * c, N);
+  }
   static constexpr int NWT = T >= 32 ? T / 32 : 1;  // warps of the team
   static constexpr int UPW = (NU + NWT - 1) / NWT;  // units per warp, at most
   float2 ucw[WLU ? UPW : 1];              // per unit: exp(i pi K / N) of the lane's group K
@@ -293,7 +302,9 @@ struct Xform {
   int lbase;                   // paired M: slot of that group's first element
   int self;                    // paired M: 0 regular, 1 group 0, 2 group N/(2 R0)
 
-  __device__ __forceinline__ void init(float2* b, const float2* t, const uint32_t* __restrict__ eb, int lane_t) {
+  // cwt: the table's CWN entries for M
+  __device__ __forceinline__ void init(float2* b, const float2* t, const float2* __restrict__ cwt,
+                                       const uint32_t* __restrict__ eb, int lane_t) {
     buf = b;
     tw = t;
     lt = lane_t;
@@ -317,7 +328,7 @@ struct Xform {
       kgrp = h ? (bb ? L - bb : L / 2) : bb;
       self = (bb == 0) ? (h == 0 ? 1 : 2) : 0;
       lbase = slot_low<PL>(kgrp);
-      cw = expi_pi(kgrp, N);
+      cw = __ldg(&cwt[kgrp]);
       p0 = p1 = pbp0 = pbp1 = 0;
     } else if constexpr (WLU) {
 #pragma unroll
@@ -325,7 +336,7 @@ struct Xform {
         int b, i;
         bool act;
         unit_of(q, b, i, act);
-        ucw[q] = expi_pi(b + (long long)E * i, N);
+        ucw[q] = __ldg(&cwt[b + E * i]);
       }
       cw = make_float2(0.f, 0.f);
       p0 = p1 = pbp0 = pbp1 = kgrp = self = lbase = g1 = 0;
@@ -335,7 +346,7 @@ struct Xform {
       p1 = slot_rest<PL>(T - 1 - Kp);
       pbp0 = pad(p0);
       pbp1 = pad(p1);
-      cw = expi_pi((long long)E * Kp, N);
+      cw = __ldg(&cwt[Kp]);
       kgrp = self = lbase = g1 = 0;
     }
     set_eps(eb);
@@ -734,8 +745,10 @@ struct Xform {
 
 // ---------------------------------------------------------------------------
 // Table set-up for one plan: access-ordered twiddles (double-precision sincospi,
-// rounded), the sign bits (SplitMix64 of seed + (j+1)*gamma, bit 63 set ->
-// eps_j = -1) and the cleared status word.
+// rounded), the sign bits of every matrix of the call (SplitMix64 of seed + (j+1)*gamma,
+// bit 63 set -> eps_j = -1) and the cleared status word.  One launch ahead of every call, so
+// its latency counts: one table entry or one sign per thread (a warp's 32 signs meet by
+// ballot), and no thread does both.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float2 root_w(long long m, long long b) {  // exp(-2 pi i m / b)
   double s, c;
@@ -743,46 +756,62 @@ __device__ __forceinline__ float2 root_w(long long m, long long b) {  // exp(-2 
   return make_float2((float)c, (float)(-s));
 }
 
+// the sign bits from block `first` on: one sign per thread
+__device__ __forceinline__ void setup_signs(uint32_t* eps, const SeedList& sl, int first) {
+  const int g = (blockIdx.x - first) * blockDim.x + threadIdx.x;
+  const int word = g >> 5;
+  if (word >= sl.count * sl.words) return;  // whole warps
+  const int i = word / sl.words;
+  const int j = (word - i * sl.words) * 32 + (threadIdx.x & 31);
+  const uint64_t z = splitmix64_mix(sl.seed[i] + (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull);
+  const uint32_t bits = __ballot_sync(0xffffffffu, j < sl.n && (z >> 63) != 0);
+  if ((threadIdx.x & 31) == 0) eps[word] = bits;
+}
+
+// Threads per block of the set-up kernels: the FP64 units do two operations per cycle and SM,
+// so the table's sincospi are spread over all SMs.
+constexpr int kSetupThreads = 32;
 template <class PL>
-__global__ void setup_kernel(float2* twt, uint32_t* eps, uint32_t* status, uint64_t seed) {
-  const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int stride = gridDim.x * blockDim.x;
-  if (tid == 0) *status = 0u;
-  for (int e = tid; e < PL::TWN; e += stride) {
-    long long m = 0, b = 1;
-    static_for<0, PL::NP - 1>([&](auto ii) {
-      constexpr int I = decltype(ii)::value;
-      constexpr int OFF = PL::tw_off(I);
-      constexpr int LEN = PL::B(I);
-      if (e >= OFF && e < OFF + LEN) {
-        const int r = e - OFF;
-        // row j, column c: pass 0 W_N^{c j} (c = thread), pass I W_B^{c j} (c = np)
-        constexpr int L = (I == 0) ? PL::T : PL::S(I);
-        int j, c;
-        if constexpr (PL::TW2) {  // [j / 2][c][j % 2]
-          j = 2 * (r / (2 * L)) + (r % 2);
-          c = (r % (2 * L)) / 2;
-        } else {                  // [j][c]
-          j = r / L;
-          c = r % L;
-        }
-        m = (long long)c * j;
-        b = (I == 0) ? PL::N : LEN;
+KD_HD constexpr int setup_table_blocks() {
+  return (PL::TWN + Xform<PL>::CWN + kSetupThreads - 1) / kSetupThreads;
+}
+
+template <class PL>
+__global__ void setup_kernel(float2* twt, uint32_t* eps, uint32_t* status, const __grid_constant__ SeedList sl) {
+  constexpr int kTableBlocks = setup_table_blocks<PL>();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *status = 0u;
+  if (blockIdx.x >= kTableBlocks) {
+    setup_signs(eps, sl, kTableBlocks);
+    return;
+  }
+  const int e = blockIdx.x * kSetupThreads + threadIdx.x;
+  if (e >= PL::TWN + Xform<PL>::CWN) return;
+  if (e >= PL::TWN) {
+    twt[e] = Xform<PL>::cw_entry(e - PL::TWN);
+    return;
+  }
+  long long m = 0, b = 1;
+  static_for<0, PL::NP - 1>([&](auto ii) {
+    constexpr int I = decltype(ii)::value;
+    constexpr int OFF = PL::tw_off(I);
+    constexpr int LEN = PL::B(I);
+    if (e >= OFF && e < OFF + LEN) {
+      const int r = e - OFF;
+      // row j, column c: pass 0 W_N^{c j} (c = thread), pass I W_B^{c j} (c = np)
+      constexpr int L = (I == 0) ? PL::T : PL::S(I);
+      int j, c;
+      if constexpr (PL::TW2) {  // [j / 2][c][j % 2]
+        j = 2 * (r / (2 * L)) + (r % 2);
+        c = (r % (2 * L)) / 2;
+      } else {                  // [j][c]
+        j = r / L;
+        c = r % L;
       }
-    });
-    twt[e] = root_w(m, b);
-  }
-  constexpr int words = (PL::N + 31) / 32;
-  for (int wd = tid; wd < words; wd += stride) {
-    uint32_t bits = 0;
-    for (int bb = 0; bb < 32; ++bb) {
-      const int j = wd * 32 + bb;
-      if (j >= PL::N) break;
-      const uint64_t z = splitmix64_mix(seed + (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull);
-      bits |= (uint32_t)(z >> 63) << bb;
+      m = (long long)c * j;
+      b = (I == 0) ? PL::N : LEN;
     }
-    eps[wd] = bits;
-  }
+  });
+  twt[e] = root_w(m, b);
 }
 
 }  // namespace kd
