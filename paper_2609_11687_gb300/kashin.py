@@ -23,6 +23,8 @@ from __future__ import annotations
 import ctypes
 import dataclasses
 import os
+import struct
+import sys
 from typing import Optional
 
 import numpy as np
@@ -301,8 +303,27 @@ def kd_rht(x, dtype, n, m, ldx, seed, inverse, y, ldy, status, stream) -> int:
 # ---------------------------------------------------------------------------
 
 def _torch():
-    import torch
-    return torch
+    t = sys.modules.get("torch")
+    if t is None:
+        import torch as t
+    return t
+
+
+# Descriptor arrays are packed from a flat list of integers: one call instead of a ctypes
+# structure per matrix (a batched call over six matrices spent 32 us here, 4 us of it in the
+# library; every field of the descriptors is eight bytes).
+_PACKERS = {}
+
+
+def _pack(fields: str, count: int, values) -> bytes:
+    key = (fields, count)
+    st = _PACKERS.get(key)
+    if st is None:
+        st = _PACKERS[key] = struct.Struct(fields * count)
+    return st.pack(*values)
+
+
+_M64 = (1 << 64) - 1
 
 
 def _dtype_code(t) -> int:
@@ -324,9 +345,13 @@ def _ld(t) -> int:
 
 
 def _stream(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is not None and torch.cuda.is_initialized():
+        return raw(torch._C._cuda_getDevice())  # the handle without a Stream object (0.2 us instead of 3)
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Workspace:
@@ -416,7 +441,7 @@ def decompose_batch(ws, iters: int, sign_seeds, layout: str = "rows", coeffs: bo
     lay = KD_VEC_ROWS if layout == "rows" else KD_VEC_COLUMNS
     n = ws[0].shape[1] if lay == KD_VEC_ROWS else ws[0].shape[0]
     dt = ws[0].dtype
-    arr = (KdMatrix * len(ws))()
+    vals = []
     res = []
     for i, w in enumerate(ws):
         if not w.is_cuda or w.dim() != 2 or w.stride(1) != 1 or w.dtype != dt:
@@ -433,11 +458,11 @@ def decompose_batch(ws, iters: int, sign_seeds, layout: str = "rows", coeffs: bo
                            centres_u=torch.empty((m, 4), **f32), centres_v=torch.empty((m, 4), **f32),
                            coeffs=torch.empty((m, 4), **f32) if coeffs else None,
                            u=None, vhat=None, resid=None, trace=None)
-        arr[i] = KdMatrix(w.data_ptr(), m, _ld(w), int(sign_seeds[i]) & ((1 << 64) - 1),
-                          _ptr(o.codes_u), _ptr(o.codes_v), _ptr(o.centres_u), _ptr(o.centres_v), _ptr(o.coeffs))
+        vals += (w.data_ptr(), m, _ld(w), int(sign_seeds[i]) & _M64, o.codes_u.data_ptr(), o.codes_v.data_ptr(),
+                 o.centres_u.data_ptr(), o.centres_v.data_ptr(), _ptr(o.coeffs) or 0)
         res.append(o)
     wsp = workspace if workspace is not None else Workspace(n, ws[0].device, count=len(ws))
-    st = kd_decompose_batch(ctypes.cast(arr, ctypes.c_void_p), len(ws), _dtype_code(dt), lay, n, int(iters),
+    st = kd_decompose_batch(_pack("QqqQQQQQQ", len(ws), vals), len(ws), _dtype_code(dt), lay, n, int(iters),
                             int(kmeans_iters), wsp.ptr, wsp.nbytes, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_decompose_batch")
@@ -490,6 +515,32 @@ def kd_matmul_2bit_bf16_batch(mats, count, batch, stream) -> int:
     return lib.kd_matmul_2bit_bf16_batch(mats, count, batch, stream)
 
 
+_FOLD_FIELDS = "QQQQQQQqqqq"  # kd_fold_mat, kd_fold_mat_f16
+
+
+def _fold_fields(decs, xs, xps, outs, b, dt, message):
+    """The fields of a product's descriptors and its outputs, the inputs checked."""
+    torch = _torch()
+    vals, res = [], []
+    for i, (d, x, xp) in enumerate(zip(decs, xs, xps)):
+        m, words = d.codes_u.shape
+        shape = x.shape
+        if len(shape) != 2 or shape[0] != b or x.dtype != dt or xp.shape != shape or xp.dtype != dt:
+            raise ValueError(message)
+        n = shape[1]
+        sx, sp = x.stride(), xp.stride()
+        ldx = sx[0] if b > 1 else n
+        if sx[1] != 1 or sp[1] != 1 or (b > 1 and sp[0] != ldx):
+            raise ValueError(message)
+        if (n + 15) // 16 != words:
+            raise ValueError("x does not match the code planes' vector length")
+        y = outs[i] if outs is not None else torch.empty((b, m), dtype=torch.float32, device=x.device)
+        vals += (d.codes_u.data_ptr(), d.codes_v.data_ptr(), d.centres_u.data_ptr(), d.centres_v.data_ptr(),
+                 x.data_ptr(), xp.data_ptr(), y.data_ptr(), n, m, ldx, _ld(y))
+        res.append(y)
+    return vals, res
+
+
 def matmul_2bit_f16(dec: "Decomposed", x, xp, out=None, stream=None):
     """kd_matmul_2bit_f16 (or _bf16): ``Y = X W_hat^T`` from the code planes on the tensor
     cores, for fp16 (or bf16) ``x`` and ``xp`` (batch, n) CUDA tensors; returns (batch, m) fp32."""
@@ -506,23 +557,10 @@ def matmul_2bit_f16_batch(decs, xs, xps, outs=None, stream=None):
     if not 1 <= len(decs) <= KD_MAX_BATCH or len(xs) != len(decs) or len(xps) != len(decs):
         raise ValueError(f"1..{KD_MAX_BATCH} matrices with one x and one xp each")
     b = xs[0].shape[0]
-    arr = (KdFoldMatF16 * len(decs))()
-    res = []
-    for i, (d, x, xp) in enumerate(zip(decs, xs, xps)):
-        m, words = d.codes_u.shape
-        if x.dim() != 2 or x.shape[0] != b or x.dtype != dt or xp.shape != x.shape \
-                or xp.dtype != x.dtype or x.stride(1) != 1 or xp.stride(1) != 1 or _ld(x) != _ld(xp):
-            raise ValueError("x and xp must be 16-bit (batch, n) tensors of one type and shape, unit inner stride")
-        n = x.shape[1]
-        if (n + 15) // 16 != words:
-            raise ValueError("x does not match the code planes' vector length")
-        y = outs[i] if outs is not None else torch.empty((b, m), dtype=torch.float32, device=x.device)
-        arr[i] = KdFoldMatF16(d.codes_u.data_ptr(), d.codes_v.data_ptr(), d.centres_u.data_ptr(),
-                              d.centres_v.data_ptr(), x.data_ptr(), xp.data_ptr(), y.data_ptr(), n, m, _ld(x),
-                              _ld(y))
-        res.append(y)
+    vals, res = _fold_fields(decs, xs, xps, outs, b, dt,
+                             "x and xp must be 16-bit (batch, n) tensors of one type and shape, unit inner stride")
     call = kd_matmul_2bit_bf16_batch if dt == torch.bfloat16 else kd_matmul_2bit_f16_batch
-    st = call(ctypes.cast(arr, ctypes.c_void_p), len(decs), b, _stream(stream))
+    st = call(_pack(_FOLD_FIELDS, len(decs), vals), len(decs), b, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_matmul_2bit_bf16_batch" if dt == torch.bfloat16 else "kd_matmul_2bit_f16_batch")
     return res
@@ -539,24 +577,26 @@ def matmul_2bit_batch(decs, xs, xps, outs=None, stream=None):
     if not 1 <= len(decs) <= KD_MAX_BATCH or len(xs) != len(decs) or len(xps) != len(decs):
         raise ValueError(f"1..{KD_MAX_BATCH} matrices with one x and one xp each")
     b = xs[0].shape[0]
-    arr = (KdFoldMat * len(decs))()
-    res = []
-    for i, (d, x, xp) in enumerate(zip(decs, xs, xps)):
-        m, words = d.codes_u.shape
-        if x.dim() != 2 or x.shape[0] != b or x.dtype != torch.float32 or xp.shape != x.shape \
-                or xp.dtype != x.dtype or x.stride(1) != 1 or xp.stride(1) != 1 or _ld(x) != _ld(xp):
-            raise ValueError("x and xp must be fp32 (batch, n) tensors of one shape, unit inner stride")
-        n = x.shape[1]
-        if (n + 15) // 16 != words:
-            raise ValueError("x does not match the code planes' vector length")
-        y = outs[i] if outs is not None else torch.empty((b, m), dtype=torch.float32, device=x.device)
-        arr[i] = KdFoldMat(d.codes_u.data_ptr(), d.codes_v.data_ptr(), d.centres_u.data_ptr(), d.centres_v.data_ptr(),
-                           x.data_ptr(), xp.data_ptr(), y.data_ptr(), n, m, _ld(x), _ld(y))
-        res.append(y)
-    st = kd_matmul_2bit_batch(ctypes.cast(arr, ctypes.c_void_p), len(decs), b, _stream(stream))
+    vals, res = _fold_fields(decs, xs, xps, outs, b, torch.float32,
+                             "x and xp must be fp32 (batch, n) tensors of one shape, unit inner stride")
+    st = kd_matmul_2bit_batch(_pack(_FOLD_FIELDS, len(decs), vals), len(decs), b, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_matmul_2bit_batch")
     return res
+
+
+def _pmat_fields(xs, outs, n, seeds):
+    """The fields of kd_pmat descriptors and the outputs, the inputs checked."""
+    torch = _torch()
+    vals, res = [], []
+    for i, x in enumerate(xs):
+        shape = x.shape
+        if x.dtype != torch.float32 or not x.is_contiguous() or len(shape) != 2 or shape[1] != n:
+            raise ValueError("inputs must be contiguous fp32 (m, n) CUDA tensors of one n")
+        y = outs[i] if outs is not None else torch.empty_like(x)
+        vals += (x.data_ptr(), y.data_ptr(), shape[0], int(seeds[i]) & _M64 if seeds is not None else 0)
+        res.append(y)
+    return vals, res
 
 
 def apply_p_batch(xs, sign_seeds, outs=None, workspace: Optional[Workspace] = None, stream=None):
@@ -566,16 +606,9 @@ def apply_p_batch(xs, sign_seeds, outs=None, workspace: Optional[Workspace] = No
     if not 1 <= len(xs) <= KD_MAX_BATCH or len(sign_seeds) != len(xs):
         raise ValueError(f"1..{KD_MAX_BATCH} matrices with one seed each")
     n = xs[0].shape[1]
-    arr = (KdPMat * len(xs))()
-    res = []
-    for i, x in enumerate(xs):
-        if x.dtype != torch.float32 or not x.is_contiguous() or x.dim() != 2 or x.shape[1] != n:
-            raise ValueError("inputs must be contiguous fp32 (m, n) CUDA tensors of one n")
-        y = outs[i] if outs is not None else torch.empty_like(x)
-        arr[i] = KdPMat(x.data_ptr(), y.data_ptr(), x.shape[0], int(sign_seeds[i]) & ((1 << 64) - 1))
-        res.append(y)
+    vals, res = _pmat_fields(xs, outs, n, sign_seeds)
     ws = workspace if workspace is not None else Workspace(n, xs[0].device, count=len(xs))
-    st = kd_apply_p_batch(ctypes.cast(arr, ctypes.c_void_p), len(xs), n, ws.ptr, ws.nbytes, _stream(stream))
+    st = kd_apply_p_batch(_pack("QQqQ", len(xs), vals), len(xs), n, ws.ptr, ws.nbytes, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_apply_p_batch")
     return res
@@ -609,15 +642,8 @@ def apply_p_prepared(xs, workspace: Workspace, outs=None, stream=None):
     if not 1 <= len(xs) <= KD_MAX_BATCH:
         raise ValueError(f"1..{KD_MAX_BATCH} matrices")
     n = xs[0].shape[1]
-    arr = (KdPMat * len(xs))()
-    res = []
-    for i, x in enumerate(xs):
-        if x.dtype != torch.float32 or not x.is_contiguous() or x.dim() != 2 or x.shape[1] != n:
-            raise ValueError("inputs must be contiguous fp32 (m, n) CUDA tensors of one n")
-        y = outs[i] if outs is not None else torch.empty_like(x)
-        arr[i] = KdPMat(x.data_ptr(), y.data_ptr(), x.shape[0], 0)
-        res.append(y)
-    st = kd_apply_p_prepared(ctypes.cast(arr, ctypes.c_void_p), len(xs), n, workspace.ptr, workspace.nbytes,
+    vals, res = _pmat_fields(xs, outs, n, None)
+    st = kd_apply_p_prepared(_pack("QQqQ", len(xs), vals), len(xs), n, workspace.ptr, workspace.nbytes,
                              _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_apply_p_prepared")
@@ -723,7 +749,7 @@ def dequantise_batch(planes, n: int, dtype=None, layout: str = "rows", outs=None
         raise ValueError(f"1..{KD_MAX_BATCH} planes")
     dtype = dtype or torch.float32
     lay = KD_VEC_ROWS if layout == "rows" else KD_VEC_COLUMNS
-    arr = (KdPlane * len(planes))()
+    vals = []
     res = []
     for i, (codes, centres) in enumerate(planes):
         m = codes.shape[0]
@@ -733,9 +759,9 @@ def dequantise_batch(planes, n: int, dtype=None, layout: str = "rows", outs=None
             o = torch.empty((m, n) if lay == KD_VEC_ROWS else (n, m), dtype=dtype, device=codes.device)
         if o.dtype != dtype:
             raise ValueError("outputs must share one dtype")
-        arr[i] = KdPlane(codes.data_ptr(), centres.data_ptr(), o.data_ptr(), m, _ld(o))
+        vals += (codes.data_ptr(), centres.data_ptr(), o.data_ptr(), m, _ld(o))
         res.append(o)
-    st = kd_dequantise_batch(ctypes.cast(arr, ctypes.c_void_p), len(planes), n, _dtype_code(dtype), lay,
+    st = kd_dequantise_batch(_pack("QQQqq", len(planes), vals), len(planes), n, _dtype_code(dtype), lay,
                              _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_dequantise_batch")
@@ -790,7 +816,7 @@ def reconstruct_batch(decs, n: int, sign_seeds, dtype=None, layout: str = "rows"
     dtype = dtype or torch.float32
     lay = KD_VEC_ROWS if layout == "rows" else KD_VEC_COLUMNS
     dev = decs[0].codes_u.device
-    arr = (KdRecMat * len(decs))()
+    vals = []
     res = []
     for i, d in enumerate(decs):
         m = d.codes_u.shape[0]
@@ -798,11 +824,11 @@ def reconstruct_batch(decs, n: int, sign_seeds, dtype=None, layout: str = "rows"
                                                          device=dev)
         if o.dtype != dtype:
             raise ValueError("outputs must share one dtype")
-        arr[i] = KdRecMat(d.codes_u.data_ptr(), d.codes_v.data_ptr(), d.centres_u.data_ptr(), d.centres_v.data_ptr(),
-                          int(sign_seeds[i]) & ((1 << 64) - 1), o.data_ptr(), m, _ld(o))
+        vals += (d.codes_u.data_ptr(), d.codes_v.data_ptr(), d.centres_u.data_ptr(), d.centres_v.data_ptr(),
+                 int(sign_seeds[i]) & _M64, o.data_ptr(), m, _ld(o))
         res.append(o)
     ws = workspace if workspace is not None else Workspace(n, dev, count=len(decs))
-    st = kd_reconstruct_batch(ctypes.cast(arr, ctypes.c_void_p), len(decs), n, _dtype_code(dtype), lay, ws.ptr,
+    st = kd_reconstruct_batch(_pack("QQQQQQqq", len(decs), vals), len(decs), n, _dtype_code(dtype), lay, ws.ptr,
                               ws.nbytes, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_reconstruct_batch")
