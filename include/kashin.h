@@ -417,8 +417,8 @@ kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, int64_t batch
  *           2-byte aligned; 16-byte aligned rows (base and ldx a multiple of 8) take
  *           128-bit loads.
  * The centres must be finite in fp16 (|c| <= 65504): a code padding past n multiplies
- * a zero input by a centre.  Every code word is read once for up to 16 batch rows, and
- * once per block of up to 256 rows beyond; the sums run in a fixed order that depends on
+ * a zero input by a centre.  Every code word is read once per block of up
+ * to 256 batch rows; the sums run in a fixed order that depends on
  * the batch size (deterministic).  A wait inside the kernel that exceeds its time limit
  * leaves NaN in the outputs it concerns.  Errors and empty calls as kd_matmul_2bit. */
 kd_status kd_matmul_2bit_f16(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,

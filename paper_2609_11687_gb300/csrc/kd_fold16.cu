@@ -5,26 +5,26 @@
 //
 // with x, xp in the 16-bit type (xp = X P from kd_apply_p, rounded by the caller), h()
 // the rounding of a centre to that type, fp32 accumulation.  Neither plane is expanded
-// in memory.  This file holds the kernel for up to 16 batch rows (decode), the argument
+// in memory.  This file holds the kernel for up to 8 batch rows (decode), the argument
 // checks and the entry points; more rows take kd_fold16_tc.cu, whose tcgen05 form decodes
-// every code once per 256 rows (7B layer: 88 us at 17 rows and 291 us at 512, where 16
-// rows at a time through this kernel took 195 us and 3.2 ms).
+// every code once per 256 rows (7B layer: 84 us at 9 to 17 rows and 286 us at 512, where 16
+// rows at a time through mma.sync took 100 us and 3.2 ms; at 8 rows and fewer it is the
+// slower one, 83 against 78 us).
 //
-// Mapping.  mma.m16n8k16 with M = the batch rows, N = 8 output channels, K = 16 inputs: each
-// code becomes its 16-bit centre in registers (kd_dec16.cuh) and feeds a B fragment
-// directly.  A work item is a tile of 32 channels (four n-tiles) of one matrix and one CTA;
-// its warps split the inputs into groups of 64 (four k-steps) round-robin, each loading the
-// next group's code words and inputs while it computes the current one, then add their
-// partial tiles in a fixed order (deterministic results).  Items are numbered longest
-// vectors first, so the hardware starts the long ones first.  Launches of at most 8 batch
-// rows skip the rows g + 8 of the A fragments (fewer registers).  Bound by the decode on
-// the ALU pipe (62 % busy at 4 rows, 7B layer, 78 us).
+// Mapping.  mma.m16n8k16 with M = the batch rows (the upper eight unused), N = 8 output
+// channels, K = 16 inputs: each code becomes its 16-bit centre in registers (kd_dec16.cuh)
+// and feeds a B fragment directly.  A work item is a tile of 32 channels (four n-tiles) of
+// one matrix and one CTA; its warps split the inputs into groups of 64 (four k-steps)
+// round-robin, each loading the next group's code words and inputs while it computes the
+// current one, then add their partial tiles in a fixed order (deterministic results).  Items
+// are numbered longest vectors first, so the hardware starts the long ones first.  Bound by
+// the decode on the ALU pipe (62 % busy at 4 rows, 7B layer).
 //
 // K order inside a group of 64 inputs.  The product is a sum over inputs, so A and B
 // may enumerate them in any common order.  In k-step j the lanes with t = lane % 4
 // take inputs 16 t + 4 j + {0, 1} for k-slots 2t, 2t+1 and 16 t + 4 j + {2, 3} for
 // k-slots 2t+8, 2t+9.  A lane's A fragments for the whole group are then its 16
-// consecutive inputs of rows g and g + 8 (g = lane / 4: two 16-byte loads per row), and
+// consecutive inputs of row g (g = lane / 4: two 16-byte loads), and
 // its B fragments are code word t of the group (inputs 16 t .. 16 t + 15) of its
 // channel: byte j of that word holds the four codes of k-step j.
 #include <cuda_runtime.h>
@@ -36,11 +36,11 @@
 namespace kd {
 namespace {
 
-// warps of a CTA, which split the inputs: eight up to 8 batch rows (two CTAs per SM; with
-// four and four, the last items of a 7B layer ran on a third of the SMs: 78 against 86 us
-// per layer at 4 rows), four beyond (the upper rows' fragments need the registers)
-__host__ __device__ constexpr int f16_warps(bool hi) { return hi ? 4 : 8; }
-constexpr int kF16Rows = 16;  // batch rows per launch (the mma's M)
+// Warps of a CTA, which split the inputs: eight (two CTAs per SM).  With four, the last items
+// of a 7B layer ran on a third of the SMs: 86 us per layer at 4 rows, 78 with eight.
+constexpr int W = 8;
+constexpr int kF16Threads = 32 * W;
+constexpr int kF16Rows = 8;   // batch rows at most
 constexpr int kF16Tile = 32;  // output channels per work item (four n-tiles)
 constexpr int kRedStride = kF16Tile + 1;
 
@@ -59,7 +59,7 @@ struct Fold16Mat {
 
 struct Fold16Params {
   int count;
-  int rows;  // batch rows of this launch (<= 16)
+  int rows;  // batch rows (<= 8)
   int64_t items;
   DecodeMul mul;
   Fold16Mat mat[KD_MAX_BATCH];
@@ -105,9 +105,8 @@ __device__ __forceinline__ void load_row16(uint32_t (&r)[8], const unsigned shor
   }
 }
 
-template <bool HI, bool BF>
-__global__ void __launch_bounds__(32 * f16_warps(HI), HI ? 3 : 2) fold16_kernel(const __grid_constant__ Fold16Params p) {
-  constexpr int W = f16_warps(HI);
+template <bool BF>
+__global__ void __launch_bounds__(kF16Threads, 2) fold16_kernel(const __grid_constant__ Fold16Params p) {
   __shared__ float red[W][kF16Rows][kRedStride];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -139,14 +138,12 @@ __global__ void __launch_bounds__(32 * f16_warps(HI), HI ? 3 : 2) fold16_kernel(
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
 
-    const bool lo_live = g < p.rows, hi_live = g + 8 < p.rows;
+    const bool row_live = g < p.rows;
     const unsigned short* xg = a.x + (int64_t)g * a.ldx;
-    const unsigned short* xh = a.x + (int64_t)(g + 8) * a.ldx;
     const unsigned short* pg = a.xp + (int64_t)g * a.ldx;
-    const unsigned short* ph = a.xp + (int64_t)(g + 8) * a.ldx;
     const int64_t groups = (a.words + 3) / 4;
     // software pipeline: the next group's code words and inputs load while this one computes
-    uint32_t wu[4], wv[4], ax[8], axh[8], ap[8], aph[8];
+    uint32_t wu[4], wv[4], ax[8], ap[8];
     auto fetch = [&](int64_t gi) {
       const int64_t wi = 4 * gi + t;  // this lane's code word of the group
       const int64_t i0 = 64 * gi + 16 * t;
@@ -156,23 +153,16 @@ __global__ void __launch_bounds__(32 * f16_warps(HI), HI ? 3 : 2) fold16_kernel(
         wu[nt] = ok ? __ldg(ru[nt] + wi) : 0u;
         wv[nt] = ok ? __ldg(rv[nt] + wi) : 0u;
       }
-      load_row16(ax, xg, i0, a.n, lo_live, a.vec);
-      load_row16(ap, pg, i0, a.n, lo_live, a.vec);
-      if constexpr (HI) {
-        load_row16(axh, xh, i0, a.n, hi_live, a.vec);
-        load_row16(aph, ph, i0, a.n, hi_live, a.vec);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) axh[k] = aph[k] = 0u;
-      }
+      load_row16(ax, xg, i0, a.n, row_live, a.vec);
+      load_row16(ap, pg, i0, a.n, row_live, a.vec);
     };
     if (warp < groups) fetch(warp);
     for (int64_t gi = warp; gi < groups; gi += W) {
-      uint32_t cwu[4], cwv[4], cax[8], caxh[8], cap[8], caph[8];
+      uint32_t cwu[4], cwv[4], cax[8], cap[8];
 #pragma unroll
       for (int k = 0; k < 4; ++k) { cwu[k] = wu[k]; cwv[k] = wv[k]; }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) { cax[k] = ax[k]; caxh[k] = axh[k]; cap[k] = ap[k]; caph[k] = aph[k]; }
+      for (int k = 0; k < 8; ++k) { cax[k] = ax[k]; cap[k] = ap[k]; }
       if (gi + W < groups) fetch(gi + W);
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt) {
@@ -184,8 +174,8 @@ __global__ void __launch_bounds__(32 * f16_warps(HI), HI ? 3 : 2) fold16_kernel(
         const uint32_t bv[8] = {vl.x, vl.y, vl.z, vl.w, vh.x, vh.y, vh.z, vh.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          mma_16<BF>(acc[nt], cax[2 * j], caxh[2 * j], cax[2 * j + 1], caxh[2 * j + 1], bu[2 * j], bu[2 * j + 1]);
-          mma_16<BF>(acc[nt], cap[2 * j], caph[2 * j], cap[2 * j + 1], caph[2 * j + 1], bv[2 * j], bv[2 * j + 1]);
+          mma_16<BF>(acc[nt], cax[2 * j], 0u, cax[2 * j + 1], 0u, bu[2 * j], bu[2 * j + 1]);
+          mma_16<BF>(acc[nt], cap[2 * j], 0u, cap[2 * j + 1], 0u, bv[2 * j], bv[2 * j + 1]);
         }
       }
     }
@@ -195,11 +185,9 @@ __global__ void __launch_bounds__(32 * f16_warps(HI), HI ? 3 : 2) fold16_kernel(
     for (int nt = 0; nt < 4; ++nt) {
       red[warp][g][8 * nt + 2 * t] = acc[nt][0];
       red[warp][g][8 * nt + 2 * t + 1] = acc[nt][1];
-      red[warp][g + 8][8 * nt + 2 * t] = acc[nt][2];
-      red[warp][g + 8][8 * nt + 2 * t + 1] = acc[nt][3];
     }
     __syncthreads();
-    for (int o = threadIdx.x; o < kF16Rows * kF16Tile; o += 32 * W) {
+    for (int o = threadIdx.x; o < kF16Rows * kF16Tile; o += kF16Threads) {
       const int r = o / kF16Tile, c = o % kF16Tile;
       if (r < p.rows && c0 + c < a.m) {
         float s = red[0][r][c];
@@ -279,13 +267,8 @@ kd_status fold16_run(const kd_fold_mat_f16* mats, int count, int64_t batch, void
   // one CTA per work item (the grid-stride loop covers grids past 2^30 items)
   const int64_t grid = items < (int64_t)1 << 30 ? items : (int64_t)1 << 30;
   const unsigned gr = (unsigned)grid;
-  if (bf) {
-    if (p.rows > 8) fold16_kernel<true, true><<<gr, 32 * f16_warps(true), 0, s>>>(p);
-    else fold16_kernel<false, true><<<gr, 32 * f16_warps(false), 0, s>>>(p);
-  } else {
-    if (p.rows > 8) fold16_kernel<true, false><<<gr, 32 * f16_warps(true), 0, s>>>(p);
-    else fold16_kernel<false, false><<<gr, 32 * f16_warps(false), 0, s>>>(p);
-  }
+  if (bf) fold16_kernel<true><<<gr, kF16Threads, 0, s>>>(p);
+  else fold16_kernel<false><<<gr, kF16Threads, 0, s>>>(p);
   if (cudaGetLastError() != cudaSuccess) return KD_ERR_CUDA;
   return KD_OK;
 }

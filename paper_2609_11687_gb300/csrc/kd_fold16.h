@@ -1,4 +1,4 @@
-// The two kernels of the 16-bit 2-bit product (kd_fold16.cu: up to 16 batch rows,
+// The two kernels of the 16-bit 2-bit product (kd_fold16.cu: up to 8 batch rows,
 // kd_fold16_tc.cu: more).
 #pragma once
 

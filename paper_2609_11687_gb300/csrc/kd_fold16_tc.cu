@@ -1,5 +1,5 @@
 // The folded 2-bit layer product of App. C for 16-bit activations on tcgen05, for more than
-// 16 batch rows (kd_fold16.cu states the product and takes fewer rows).  The code planes
+// 8 batch rows (kd_fold16.cu states the product and takes fewer rows).  The code planes
 // are read and decoded once per block of up to 256 batch rows.
 //
 // Mapping.  tcgen05.mma with M = 128 output channels, N = the batch rows of the block,
@@ -27,8 +27,8 @@
 // in rank order.  The split follows from the batch alone, so a matrix gives the same bits
 // alone and in a batched call.
 //
-// Measured (7B layer): 88 / 98 / 129 / 159 / 291 us at 17 / 64 / 128 / 256 / 512 rows; at 512
-// rows that is 1.43 PFLOP/s, 74 % of the measured bf16 rate.  The MMA thread branches on
+// Measured (7B layer): 84 / 96 / 122 / 155 / 286 us at 9 to 17 / 64 / 128 / 256 / 512 rows; at
+// 512 rows that is 1.45 PFLOP/s, 75 % of the measured bf16 rate.  The MMA thread branches on
 // elect.sync (kd_tc.cuh): with a lane test instead, every tcgen05 instruction cost a loop
 // over the lanes and 512 rows took 422 us.
 #include <cuda_runtime.h>
@@ -447,6 +447,7 @@ cudaError_t launch_tc(FoldTcParams& p, int64_t tiles, cudaStream_t s) {
 template <bool BF>
 cudaError_t launch_tc(FoldTcParams& p, int64_t tiles, bool tma, cudaStream_t s) {
   if (!tma) return p.nt <= 64 ? launch_tc<BF, 64, false>(p, tiles, s) : launch_tc<BF, 256, false>(p, tiles, s);
+  if (p.nt <= 16) return launch_tc<BF, 16, true>(p, tiles, s);
   if (p.nt <= 32) return launch_tc<BF, 32, true>(p, tiles, s);
   if (p.nt <= 64) return launch_tc<BF, 64, true>(p, tiles, s);
   if (p.nt <= 128) return launch_tc<BF, 128, true>(p, tiles, s);

@@ -118,31 +118,30 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 }
 
 // Bounded wait for the phase of `bar` with this parity: false, with *fail set, once a wait of
-// this CTA has taken longer than kWaitCycles (every later one then gives up at once).  The
-// suspend-time hint (10 ms) lets the hardware park the thread: polling took a tenth of the
-// issue slots from the decoding warps.
+// this CTA has taken kWaitTries tries (every later one then gives up at once).  A try parks the
+// thread for some hundred cycles at most, so the limit is near a second.  The loop is a try, a
+// counter and two branches: with a clock and a flag read in it, polling took a fifth of the
+// instructions of the whole kernel.
+constexpr uint32_t kWaitTries = 1u << 22;
 __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* fail) {
-  auto parked = [&]() {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity), "r"(10000000u)
-        : "memory");
-    return done != 0;
-  };
-  if (parked()) return true;
-  const long long t0 = clock64();
-  while (!parked()) {
-    if (*(volatile int*)fail) return false;
-    if (clock64() - t0 > kWaitCycles) {
-      *(volatile int*)fail = 1;
-      return false;
-    }
-  }
-  return true;
+  if (mbar_try_wait(bar, parity)) return true;
+  if (*(volatile int*)fail) return false;
+  uint32_t left = kWaitTries;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "TRY_%=:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra DONE_%=;\n\t"
+      "add.u32 %0, %0, -1;\n\t"
+      "setp.ne.u32 q, %0, 0;\n\t"
+      "@q bra TRY_%=;\n\t"
+      "DONE_%=:\n\t}"
+      : "+r"(left)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  if (left != 0) return true;
+  *(volatile int*)fail = 1;
+  return false;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -1,4 +1,4 @@
-"""The 16-bit product from the 2-bit planes for more than 16 batch rows (tcgen05), against
+"""The 16-bit product from the 2-bit planes for more than 8 batch rows (tcgen05), against
 the fp64 oracle on the same 16-bit inputs and centres.
 
 Sizes sit at the edges of its tiles: 128 channels, 128 inputs per unit, accumulations of 8
@@ -18,6 +18,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("n,m,batch,bf16", [
+    (100, 30, 9, True),        # the fewest rows, one unit per plane
+    (4096, 128, 16, False),    # a full block of 16 rows
     (16, 1, 17, False),        # half a unit, three of the four CTAs of a cluster idle
     (128, 128, 64, True),      # one unit per plane, one full tile
     (1000, 129, 65, False),    # a partial code word, unaligned code rows, a second tile of one channel
