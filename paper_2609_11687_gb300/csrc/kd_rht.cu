@@ -283,17 +283,15 @@ __device__ __forceinline__ void transform_and_store(const RhtParams& p, float2 (
   }
 }
 
-// sign bits of the vector, once per CTA (entry j: bit j % 32 of word j / 32)
+// sign bits of the vector, once per CTA (entry j: bit j % 32 of word j / 32): one sign per
+// lane, a warp's 32 signs meet by ballot
 __device__ __forceinline__ void stage_sign_bits(uint32_t* sbits, int64_t n, uint64_t seed, int nthreads) {
   const int words = (int)((n + 31) / 32);
-  for (int wd = threadIdx.x; wd < words; wd += nthreads) {
-    uint32_t bits = 0;
-    for (int bb = 0; bb < 32; ++bb) {
-      const int64_t j = (int64_t)wd * 32 + bb;
-      if (j >= n) break;
-      bits |= (uint32_t)(splitmix64_mix(seed + (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull) >> 63) << bb;
-    }
-    sbits[wd] = bits;
+  for (int wd = threadIdx.x >> 5; wd < words; wd += nthreads >> 5) {
+    const int j = wd * 32 + (threadIdx.x & 31);
+    const uint64_t z = splitmix64_mix(seed + (uint64_t)(j + 1) * 0x9E3779B97F4A7C15ull);
+    const uint32_t bits = __ballot_sync(0xffffffffu, j < n && (z >> 63) != 0);
+    if ((threadIdx.x & 31) == 0) sbits[wd] = bits;
   }
 }
 
@@ -426,12 +424,12 @@ __global__ void __launch_bounds__(rht_threads(LOG_B), rht_min_blocks(LOG_B)) rht
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) mbar_init(&mbar[s], 1);
     mbar_init_fence();
+    // the first copies before the signs: drawing n of them in every CTA takes 2 to 6 us of a
+    // launch (n = 4096 to 11008), in which the copies land (7B layer 260 -> 256 us)
+    for (int64_t i = 0; i < STAGES && i < n_iter; ++i) issue(i, (int)i);
   }
   stage_sign_bits(sbits, p.n, p.seed, THREADS);
   __syncthreads();
-  if (tid == 0) {
-    for (int64_t i = 0; i < STAGES && i < n_iter; ++i) issue(i, (int)i);
-  }
 
   // this team's unit, walked as (vector j, block bi) without a division per unit
   const int64_t dj = per_iter / nblk, db = per_iter - dj * nblk;
