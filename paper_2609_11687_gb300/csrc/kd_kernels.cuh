@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(PL::THREADS, PL::MINB) decompose_kernel(DecPar
   const int team = threadIdx.x / T;
   const int lt = threadIdx.x - team * T;
   const float2* tw;
-  constexpr bool QUICK = PL::N < 4096;  // launches short enough for their start to count
+  constexpr bool QUICK = QuickStart<PL>::value;
   float2* buf = cta_setup<PL, QUICK>(smem, p.twt, tw, team);
   float2* red = buf + PL::BUF;
   Xform<PL> xf;

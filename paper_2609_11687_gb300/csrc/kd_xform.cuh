@@ -93,6 +93,16 @@ struct PackedRoots {
   static constexpr bool value = false;
 };
 
+// Decompose kernels that read M's roots from the table and stage the table 16 bytes a load: the
+// short lengths, whose launches are short enough for 3 us of start-up to count (300 vectors of
+// 1024: 61.8 to 55.8 us).  In the others the compiler arranges the block loop better without it:
+// whole launches 0.6 % at n = 4096, 1.5 % at 11008, and at 128 60,000 vectors 409 us against 416
+// (412 before; 300 vectors 47.4 against 45.5, 49.6 before).
+template <class PL>
+struct QuickStart {
+  static constexpr bool value = PL::N < 4096 && PL::N != 128;
+};
+
 template <int N_, int T_, int Q_, int UMODE_, int MINB_, int... Rs>
 struct Plan {
   static constexpr int N = N_;
