@@ -314,10 +314,10 @@ def run_gpu(args) -> dict:
     wsb = {n_: kd.Workspace(n_, dev, count=len(ix)) for n_, ix in groups.items()}
     stream = torch.cuda.current_stream()
 
-    # kernels per step: batch = set-up + sign sets + decompose per length; single =
-    # set-up + decompose per matrix (longer lengths always run one launch per matrix)
+    # kernels per step: batch = set-up + decompose per length; single = the same per
+    # matrix (longer lengths always run one launch per matrix)
     if args.launch == "batch":
-        launches_per_step = sum((3 if len(ix) > 1 else 2) if kd.kd_batchable(n_) else 2 * len(ix)
+        launches_per_step = sum(2 if kd.kd_batchable(n_) else 2 * len(ix)
                                 for n_, ix in groups.items())
     else:
         launches_per_step = 2 * len(layer0)
@@ -630,14 +630,15 @@ def measure_inference(kd, torch, layer, iters, wss, stream):
                        "achieved": round(deq_bytes / (ms_deq / 1e3) / 1e9, 1), "peak": hbm, "unit": "GB/s",
                        "frac": round(deq_bytes / (ms_deq / 1e3) / 1e9 / hbm, 4), "peak_basis": basis,
                        "algorithmic_bytes_per_param": 4.5},
-        "matmul_2bit": {"kernel": "fold_kernel (Y = X U_q^T + XP V_q^T from the 2-bit planes: one "
-                                  "kd_matmul_2bit_batch per layer and group of up to 2 rows; XP by one "
+        "matmul_2bit": {"kernel": "fold_kernel (1 row) / fold_tc_kernel (2 rows and more: tcgen05, fp32 inputs as three "
+                                  "bf16 pieces; Y = X U_q^T + XP V_q^T from the 2-bit planes: one "
+                                  "kd_matmul_2bit_batch per layer; XP by one "
                                   "kd_apply_p_prepared per vector length on tables kd_prepare_p derived once "
                                   "per layer; ms_xp_deriving_tables: kd_apply_p_batch, tables derived per call) "
                                   "against torch.matmul fp16 on W_hat "
-                                  "(cuBLAS, one call per matrix), whole layer; f16_tc: fold16_kernel "
-                                  "(kd_matmul_2bit_f16_batch, fp16 X and XP, mma.sync m16n8k16 with fp32 sums, "
-                                  "one launch per 16 rows); L2 flushed before every repetition, median",
+                                  "(cuBLAS, one call per matrix), whole layer; f16_tc: fold16_kernel (up to 8 rows, "
+                                  "mma.sync m16n8k16) / fold16_tc_kernel (more rows, tcgen05): "
+                                  "kd_matmul_2bit_f16_batch, fp16 X and XP, fp32 sums; L2 flushed before every repetition, median",
                         "algorithmic_bytes": "codes 0.5 B per weight + centres + x, XP, y", "peak_basis": basis,
                         **folded},
     }
@@ -849,33 +850,35 @@ def run_profile_case(args) -> None:
         log(f"[profile-case] ok: {args.profile_kernel} n={spec.N} m={spec.M}")
         return
     if args.profile_kernel == "fold":
-        # the layer's 2-bit products at batch 1 (one kd_matmul_2bit_batch), three times
+        # the layer's 2-bit products (one kd_matmul_2bit_batch, 1 row by default), three times
+        rows = args.profile_rows or 1
         decs = []
         for s_ in layer_fn(0):
             w_ = synth.generate(s_, device="cuda")
             decs.append((s_, kd.decompose(w_, args.iters, s_.sign_seed)))
             del w_
-        xs = {n: torch.randn((1, n), device="cuda") for n in {s_.N for s_, _ in decs}}
+        xs = {n: torch.randn((rows, n), device="cuda") for n in {s_.N for s_, _ in decs}}
         xps = [kd.apply_p(xs[s_.N], s_.sign_seed) for s_, _ in decs]
         for _ in range(3):
             kd.matmul_2bit_batch([d for _, d in decs], [xs[s_.N] for s_, _ in decs], xps)
         torch.cuda.synchronize()
-        log("[profile-case] ok: fold, 7B layer, batch 1")
+        log(f"[profile-case] ok: fold, 7B layer, batch {rows}")
         return
     if args.profile_kernel == "fold16":
-        # the layer's fp16 tensor-core products at batch 4 (one kd_matmul_2bit_f16_batch), three times
+        # the layer's fp16 products (one kd_matmul_2bit_f16_batch, 4 rows by default), three times
+        rows = args.profile_rows or 4
         decs = []
         for s_ in layer_fn(0):
             w_ = synth.generate(s_, device="cuda")
             decs.append((s_, kd.decompose(w_, args.iters, s_.sign_seed)))
             del w_
-        xs = {n: torch.randn((4, n), device="cuda") for n in {s_.N for s_, _ in decs}}
+        xs = {n: torch.randn((rows, n), device="cuda") for n in {s_.N for s_, _ in decs}}
         xps = [kd.apply_p(xs[s_.N], s_.sign_seed).half() for s_, _ in decs]
         x16 = {n: x.half() for n, x in xs.items()}
         for _ in range(3):
             kd.matmul_2bit_f16_batch([d for _, d in decs], [x16[s_.N] for s_, _ in decs], xps)
         torch.cuda.synchronize()
-        log("[profile-case] ok: fold16, 7B layer, batch 4")
+        log(f"[profile-case] ok: fold16, 7B layer, batch {rows}")
         return
     if args.profile_kernel == "rht":
         y = torch.empty(w.shape, dtype=torch.float32, device="cuda")
@@ -910,6 +913,7 @@ def main():
     ap.add_argument("--skip-e2e", action="store_true")
     ap.add_argument("--profile-case", action="store_true", help="small single-matrix case for ncu")
     ap.add_argument("--profile-m", type=int, default=32768)
+    ap.add_argument("--profile-rows", type=int, default=0, help="batch rows of the fold cases (0 = their default)")
     ap.add_argument("--profile-matrix", type=int, default=0, help="layer matrix index (0 = q, 6 = down)")
     ap.add_argument("--profile-kernel", default="decompose", choices=["decompose", "rht", "reconstruct", "dequantise", "fold", "fold16"])
     args = ap.parse_args()

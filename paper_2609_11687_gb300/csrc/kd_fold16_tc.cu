@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
           const uint64_t db = db0 + (uint64_t)(s * (bbytes >> 4)) + (BH == 2 ? h * (bstage >> 4) : 0u);
 #pragma unroll
           for (int q = 0; q < kStageK / 16; ++q)
-            tc_mma_ta(d, ta + 32 * h + 8 * q, db + 2 * q, idesc, !fresh || h + q != 0);
+            tc_mma(d, ta + 32 * h + 8 * q, db + 2 * q, idesc, !fresh || h + q != 0);
           if (BH == 1 || h == 1) tc_commit(&ctl.empty_b[s]);
           if (h == 1) {
             tc_commit(&ctl.empty_a[sa]);

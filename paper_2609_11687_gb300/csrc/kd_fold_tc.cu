@@ -32,7 +32,7 @@
 // in the centres) cannot be split or summed without their weights: their outputs are summed
 // again by plain fp32 FMAs.
 //
-// Measured (7B layer, L2 cold): 116 us at 2 rows, 126 at 16, 429 at 64; the table-lookup
+// Measured (7B layer, L2 cold): 120 us at 2 rows, 131 at 16, 448 at 64; the table-lookup
 // kernel took 121 us per two rows (970 at 16).  Error against 64 bits at 16 rows, 2-norm:
 // 6e-8 to 8e-8, against 1.6e-7 to 2.2e-7 before (1.0e-7 with centres that are not
 // symmetric).  The ALU pipe is 68 % busy with the decode and the split of the inputs.
@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
         for (int pn = 0; pn < 2; ++pn)
 #pragma unroll
           for (int q = 0; q < kStageK / 16; ++q)
-            tc_mma_ta(tmem + pn * 64, ta + pn * 32 + 8 * q, db + 2 * q, idesc, in_chunk != 0 || q != 0);
+            tc_mma(tmem + pn * 64, ta + pn * 32 + 8 * q, db + 2 * q, idesc, in_chunk != 0 || q != 0);
         tc_commit(&ctl.empty_a[sa]);
         tc_commit(&ctl.empty_b[sb]);
         if (end) tc_commit(&ctl.acc_full);

@@ -30,7 +30,7 @@
 // for M, the greedy steps in shared memory, 288 instructions per element and P, half the
 // shared-memory wavefronts conflicts) and now:
 //   n = 640 x 8000 2.75 -> 1.91 ms, 2560 x 6000 4.92 -> 3.29, 5120 x 5120 (columns, 3
-//   refinements) 8.04 -> 5.98, 10000 x 2000 9.59 -> 6.24, 12288 x 2000 9.68 -> 6.35,
+//   refinements) 8.04 -> 5.92, 10000 x 2000 9.59 -> 6.24, 12288 x 2000 9.68 -> 6.35,
 //   13824 x 2000 12.73 -> 9.94.
 // Every result keeps its bits: the same operations on the same values in the same order.
 //
