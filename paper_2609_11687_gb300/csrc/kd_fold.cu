@@ -9,7 +9,7 @@
 //
 // This file holds the argument checks, the entry points and the kernel for one batch row;
 // two rows and more take kd_fold_tc.cu, on the tensor cores, 16 rows in one pass over the
-// codes (7B layer: 120 us at 2 rows and 131 at 16, where this kernel, two rows at a time,
+// codes (7B layer: 116 us at 2 rows and 131 at 16, where this kernel, two rows at a time,
 // took 121 and 970; at one row it takes 85).
 //
 // Mapping.  One launch serves up to KD_MAX_BATCH matrices (a layer): persistent CTAs

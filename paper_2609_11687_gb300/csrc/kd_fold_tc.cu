@@ -13,9 +13,10 @@
 // sum of a few hundred of them); every kChunk stages the sums move to fp32 registers.
 //
 // Mapping.  tcgen05.mma with M = 128 output channels, N = 3 values per batch row (16 rows per
-// block), K = the inputs in stages of 64.  A cluster of two CTAs owns a tile of 128 channels:
-// CTA 0 the u plane with x, CTA 1 the v plane with xp; their sums are added at the end over
-// distributed shared memory.  In a CTA
+// block), K = the inputs in stages of 64.  A cluster owns a tile of 128 channels: half of its
+// CTAs the u plane with x, half the v plane with xp, each a part of the inputs (two parts up to
+// 16 rows, one beyond); their sums are added at the end over distributed shared memory.  In a
+// CTA
 //  * two groups of four warps decode, every other stage each: a thread turns the four code
 //    words of its channel into its TMEM lane of either plane (the MMA takes A from TMEM:
 //    through shared memory, the planes' writes and reads filled its bandwidth and 16 rows of
@@ -32,7 +33,7 @@
 // in the centres) cannot be split or summed without their weights: their outputs are summed
 // again by plain fp32 FMAs.
 //
-// Measured (7B layer, L2 cold): 120 us at 2 rows, 131 at 16, 448 at 64; the table-lookup
+// Measured (7B layer, L2 cold): 116 us at 2 rows, 131 at 16, 448 at 64; the table-lookup
 // kernel took 121 us per two rows (970 at 16).  Error against 64 bits at 16 rows, 2-norm:
 // 6e-8 to 8e-8, against 1.6e-7 to 2.2e-7 before (1.0e-7 with centres that are not
 // symmetric).  The ALU pipe is 68 % busy with the decode and the split of the inputs.
@@ -74,6 +75,7 @@ struct FoldTcParams {
   int count;
   int rows;        // batch rows of the call
   int row_blocks;  // blocks of kRows rows
+  int split;       // parts of each plane's inputs, one CTA each
   DecodeMul mul;
   FoldTcMat mat[KD_MAX_BATCH];
 };
@@ -102,8 +104,10 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   const int lane = threadIdx.x & 31;
 
-  const uint32_t pl = cluster_rank();  // 0: u plane and x, 1: v plane and xp
-  const uint32_t id = blockIdx.x / 2;
+  const uint32_t rank = cluster_rank(), split = (uint32_t)p.split;
+  const uint32_t pl = rank >= split;  // 0: u plane and x, 1: v plane and xp
+  const uint32_t part = rank - pl * split;
+  const uint32_t id = blockIdx.x / (2 * split);
   const uint32_t tile = id / (uint32_t)p.row_blocks;
   const int row0 = (int)(id - tile * p.row_blocks) * kRows;
   int mi = 0;
@@ -112,16 +116,20 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   const int64_t c0 = (int64_t)(tile - p.tile0[mi]) * kTile;
   const int rows = p.rows - row0 < kRows ? p.rows - row0 : kRows;
   const int nt = (3 * rows + 15) / 16 * 16;
-  const int L = (int)((a.n + kStageK - 1) / kStageK);  // stages
+  // this CTA's part of the inputs: n inputs from n0, in L stages (none where n < 64 split)
+  const uint32_t all = (uint32_t)((a.n + kStageK - 1) / kStageK);
+  const int s0 = (int)(all * part / split), L = (int)(all * (part + 1) / split) - s0;
+  const int64_t n0 = (int64_t)kStageK * s0;
+  const int n = (int)(a.n - n0 < (int64_t)kStageK * L ? a.n - n0 : (int64_t)kStageK * L);
 
   // decoding threads: channel r of the tile, its centres, its first code words
   const int grp = warp >> 2;
   const int r = threadIdx.x & (kTile - 1);
   const bool live = warp < kDecWarps && c0 + r < a.m;
-  const uint32_t* code_row = a.codes[pl] + (live ? c0 + r : 0) * a.words;
-  const int words = live ? (int)a.words : 0;
+  const uint32_t* code_row = a.codes[pl] + (live ? c0 + r : 0) * a.words + 4 * s0;
+  const int words = live ? (n + 15) / 16 : 0;
   const bool vec = a.vec_codes;
-  auto fetch = [&](int st) -> uint4 {  // the words of stage st (of either pass), zero past the row and m
+  auto fetch = [&](int st) -> uint4 {  // the words of stage st (of either pass), zero past the part and m
     const int s = st < L ? st : st - L;
     const int w0 = 4 * s;
     const int left = words - w0;
@@ -211,12 +219,12 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
     const int sg = (warp - kDecWarps) >> 1;
     const int t = threadIdx.x & 63;
     const int seg = t & 7, br0 = t >> 3;
-    const float* src = a.x[pl] + (int64_t)(row0 + br0) * a.ldx + 8 * seg;
+    const float* src = a.x[pl] + (int64_t)(row0 + br0) * a.ldx + n0 + 8 * seg;
     const bool vec_x = a.vec_x;
     uint32_t big[2] = {0u, 0u};
     auto load = [&](int st, float (&v)[2][8]) {
       const int i0 = kStageK * (st < L ? st : st - L);
-      const int left = (int)(a.n - i0 - 8 * seg);
+      const int left = n - i0 - 8 * seg;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const float* q = src + 8 * h * a.ldx + i0;
@@ -292,7 +300,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       const int pass = done / chunks, c = done - pass * chunks;
       done_stage = pass * L + (c + 1 < chunks ? (c + 1) * kChunk : L);
     };
-    next_end();
+    if (chunks > 0) next_end();
     auto promote = [&]() {
       ctl_wait(ctl, &ctl.acc_full, done & 1);
       tc_fence_after();
@@ -371,10 +379,10 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       float v = acc[k];
       if (c < rows && (plain_channel || ((plain >> c) & 1))) {
         v = 0.f;
-        const float* q = a.x[pl] + (int64_t)(row0 + c) * a.ldx;
+        const float* q = a.x[pl] + (int64_t)(row0 + c) * a.ldx + n0;
         const float cc[4] = {cen.x, cen.y, cen.z, cen.w};
-        for (int64_t i = 0; live && i < a.n; ++i) {
-          const uint32_t code = (__ldg(code_row + (i >> 4)) >> (2 * (int)(i & 15))) & 3u;
+        for (int i = 0; live && i < n; ++i) {
+          const uint32_t code = (__ldg(code_row + (i >> 4)) >> (2 * (i & 15))) & 3u;
           const float ce = (code & 2u) ? ((code & 1u) ? cc[3] : cc[2]) : ((code & 1u) ? cc[1] : cc[0]);
           v = __fmaf_rn(ce, __ldg(q + i), v);
         }
@@ -383,11 +391,13 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
     }
   }
   cluster_sync_all();
-  // CTA 0 writes the even batch rows, CTA 1 the odd ones: u plane first
+  // the CTAs share the batch rows; parts in order, the u plane's first
   if (live) {
-    for (int c = 2 * grp + (int)pl; c < rows; c += 4) {
+    for (int c = 2 * (int)rank + grp; c < rows; c += 4 * (int)split) {
       const uint32_t at = ring + (c * kTile + r) * 4;
-      a.y[(int64_t)(row0 + c) * a.ldy + c0 + r] = __fadd_rn(ld_dsmem(at, 0), ld_dsmem(at, 1));
+      float v = ld_dsmem(at, 0);
+      for (uint32_t q = 1; q < 2 * split; ++q) v = __fadd_rn(v, ld_dsmem(at, q));
+      a.y[(int64_t)(row0 + c) * a.ldy + c0 + r] = v;
     }
   }
   cluster_sync_all();  // the peer's reads of this CTA's shared memory are done
@@ -416,6 +426,12 @@ kd_status fold_tc_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStr
     FoldTcParams p;
     p.rows = (int)(batch - b0 < kMaxRows ? batch - b0 : kMaxRows);
     p.row_blocks = (p.rows + kRows - 1) / kRows;
+    // Up to one row block, two parts per plane: a small layer's tiles alone leave places idle
+    // (16 rows: one 4096 x 11008 matrix 78 -> 44 us, a 768-wide layer's six 27 -> 19), and the
+    // 7B layer takes the same (119 -> 116 us at 2 rows, 130 at 16).  Four parts were slower
+    // (7B layer 159 us at 16 rows), and with more row blocks two already are (17 rows: 222 ->
+    // 238).  Not by the number of tiles: a matrix's results do not depend on the others'.
+    p.split = p.rows <= kRows ? 2 : 1;
     p.count = 0;
     int64_t tiles = 0;
     for (int i = 0; i < count; ++i) {
@@ -441,13 +457,13 @@ kd_status fold_tc_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStr
     }
     if (tiles == 0) return KD_OK;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(tiles * p.row_blocks * 2));
+    cfg.gridDim = dim3((unsigned)(tiles * p.row_blocks * 2 * p.split));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.x = (unsigned)(2 * p.split);
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;

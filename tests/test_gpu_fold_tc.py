@@ -44,6 +44,8 @@ def _case(kd, n, m, batch, kmeans=0, seed=0):  # noqa: F811
     (64, 128, 16),     # one full stage, tile and block
     (1000, 129, 17),   # a partial code word, unaligned code rows, a second tile and block of one
     (2048, 127, 3),    # exactly one accumulation
+    (4160, 130, 16),   # parts of 32 and 33 stages: an accumulation of one stage ends a part
+    (1000, 19, 6),     # a partial code word and unaligned code rows in the second part
     (2112, 130, 5),    # one stage into the second
     (11008, 128, 33),  # six accumulations, three blocks
     (16384, 40, 9),
