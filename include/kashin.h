@@ -373,9 +373,12 @@ kd_status kd_measure_fp32_peak(double* tflops, void* stream);
  *   xp                 device fp32, the same rows times P (kd_apply_p with the matrix's
  *                      sign seed on the rows of X), same layout and ldx.
  *   y                  device fp32, batch rows of m outputs, row r at y + r*ldy (ldy >= m).
- * Every code word is read once per group of up to 16 batch rows; nothing is rounded below
- * fp32, and the sums run in a fixed order (deterministic).  A wait inside the kernel that
- * exceeds its time limit leaves NaN in the outputs it concerns.  Errors: KD_ERR_INVALID_ARG (sizes, null or
+ * Every code word is read once per group of up to 16 batch rows; the sums run in a fixed
+ * order that depends on the batch size (deterministic).  With two rows and more an input is
+ * taken to 2^-32 of the largest magnitude of its row (or of either half of the row) and the
+ * sums of the inputs of one code are exact; every other operation is fp32.  y holds scratch
+ * values until the call's last kernel has written it, and must not overlap the inputs.  A wait
+ * inside the kernel that exceeds its time limit leaves NaN in the outputs it concerns.  Errors: KD_ERR_INVALID_ARG (sizes, null or
  * unaligned pointers when m > 0 and batch > 0), KD_ERR_CUDA (launch).  m == 0 or
  * batch == 0 enqueues nothing. */
 kd_status kd_matmul_2bit(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,

@@ -1,18 +1,23 @@
 // The folded 2-bit layer product of App. C in fp32 (kd_fold.cu states it) on the tensor
 // cores, for two batch rows and more, with nothing rounded to 16 bits.
 //
-//  * An input is the exact sum of three bf16 values, x = x1 + x2 + x3 (truncated to 8
-//    significant bits, the rest, and what that leaves: 24 bits).
+//  * An input is a fixed-point number on the grid of its row (of this CTA's part of it): with
+//    2^k the power of two above the row's largest magnitude, x = 2^k (d1 + d2 + d3 + d4), where
+//    d1, d2, d3 are the digits of weight 2^-7, 2^-15, 2^-23 (at most 128 of each, exact in bf16)
+//    and d4, below 2^-24, is cut to bf16: 32 bits below the row's largest.
 //  * A weight enters as which code it has, not as its centre: with T_q the sum of the inputs
 //    whose code is q, the product of one plane is c0 T0 + c1 T1 + c2 T2 + c3 T3.  The MMAs
 //    multiply the inputs by planes of -1, 0 and 1, which are exact in bf16:
 //        D_in = T2 - T1, D_out = T3 - T0, and where a channel of the tile has centres that are
 //        not symmetric about 0 (after k-means refinement), E_in = T1 + T2, E_out = T0 + T3.
 //    The centres stay fp32 and multiply the sums.
-// Products are exact, and so are most additions inside the tensor core (an 8-bit value and a
-// sum of a few hundred of them); every kChunk stages the sums move to fp32 registers.
+// The sums of d1, d2 and d3 are whole numbers of at most 24 bits for up to 2^17 inputs, so the
+// tensor core, which cuts each addition off instead of rounding it, adds them exactly; kChunk
+// bounds an accumulation.  Pieces taken from the floating-point bits of each input instead
+// (8 + 8 + 8) lost up to 2^-24 of the running sum per addition: a row led by one input erred by
+// 4.7e-6 of its norm, log-normal inputs by 2.3e-6, and inputs below 2^-110 lost their last bits.
 //
-// Mapping.  tcgen05.mma with M = 128 output channels, N = 3 values per batch row (16 rows per
+// Mapping.  tcgen05.mma with M = 128 output channels, N = 4 digits per batch row (16 rows per
 // block), K = the inputs in stages of 64.  A cluster owns a tile of 128 channels: half of its
 // CTAs the u plane with x, half the v plane with xp, each a part of the inputs (two parts up to
 // 16 rows, one beyond); their sums are added at the end over distributed shared memory.  In a
@@ -21,22 +26,26 @@
 //    words of its channel into its TMEM lane of either plane (the MMA takes A from TMEM:
 //    through shared memory, the planes' writes and reads filled its bandwidth and 16 rows of
 //    the 7B layer took 190 us);
+//  * the rows' largest magnitudes come from a small launch ahead (row_grid_kernel); where an
+//    infinity or a NaN is among a row, all warps first look through the tile's rows for them;
 //  * two groups of two warps split the inputs into the B tile in shared memory, every other
-//    stage each, their loads two own stages ahead (the inputs come from L2);
+//    stage each, their loads two own stages ahead (again from L2; packed additions, so that
+//    the decode has the ALU pipe);
 //  * one thread issues the MMAs;
 //  * the decoding warps also move finished sums from TMEM to registers.
 // With centres that are not symmetric the K loop runs twice, over the D and then the E planes.
 // TMEM (256 of 512 columns, two CTAs per SM): the sums of two planes, and one slot of A for
 // each decoding group; while one CTA waits for its slot or its sums, the other decodes.
 //
-// Rows and channels with an infinity, a NaN or a magnitude of 2^101 and more (in the inputs,
-// in the centres) cannot be split or summed without their weights: their outputs are summed
-// again by plain fp32 FMAs.
+// An infinity among the inputs counts as zero there and is added with its centre at the end;
+// a NaN makes its row NaN.  Channels with a centre of 2^101 and more, an infinity or a NaN
+// among them (their products with a plain sum could overflow), and rows of more infinities
+// than are noted, are summed again by plain fp32 FMAs.
 //
-// Measured (7B layer, L2 cold): 116 us at 2 rows, 131 at 16, 448 at 64; the table-lookup
-// kernel took 121 us per two rows (970 at 16).  Error against 64 bits at 16 rows, 2-norm:
-// 6e-8 to 8e-8, against 1.6e-7 to 2.2e-7 before (1.0e-7 with centres that are not
-// symmetric).  The ALU pipe is 68 % busy with the decode and the split of the inputs.
+// Measured (7B layer, L2 cold): 121 us at 2 rows, 140 at 16, 467 at 64; the table-lookup
+// kernel takes 125 us per two rows (981 at 16).  Error against 64 bits, 2-norm: 5e-8 to 6e-8 (8e-8
+// with centres that are not symmetric) for normal, all-positive, log-normal and very small inputs
+// and rows led by one, n = 256 to 16384; the table-lookup kernel has 9e-8 to 2.9e-7.
 #include <cuda_runtime.h>
 
 #include "kashin.h"
@@ -50,15 +59,21 @@ namespace {
 constexpr int kTile = 128;     // output channels per CTA (the MMA's M, the TMEM lanes)
 constexpr int kRows = 16;      // batch rows per block
 constexpr int kStageK = 64;    // inputs per stage
-constexpr int kChunk = 32;     // stages per TMEM accumulation
+constexpr int kDigits = 4;     // bf16 digits per input
+constexpr int kChunk = 1024;   // stages per TMEM accumulation (2^16 inputs)
 constexpr int kDecWarps = 8;   // decoding warps: two groups of four
 constexpr int kSplitWarps = 4;  // two groups of two
 constexpr int kThreads = 32 * (kDecWarps + kSplitWarps + 1);
 constexpr int kSlotsA = 2, kSlotsB = 4;    // A in TMEM, B in shared memory
-constexpr int kBBytes = 3 * kRows * 128;
+constexpr int kBBytes = kDigits * kRows * 128;
 constexpr int kSmem = kSlotsB * kBBytes + 1024;
 constexpr uint32_t kCols = 256;            // TMEM: sums of plane p at 64 p, A slot s at 128 + 64 s (32 per plane)
 constexpr uint32_t kBig = 0x72000000u;     // bits of 2^101
+constexpr uint32_t kInf = 0x7F800000u;
+constexpr int kTopExp = 100;               // the sums take at most 2^100 of the row's 2^k before the centres
+constexpr int kInfs = 64;                  // infinities noted per CTA
+constexpr int kGridThreads = 256;          // of row_grid_kernel
+constexpr int kScan = 8;                   // loads in flight per thread of the search for the rows' largest
 
 struct FoldTcMat {
   const uint32_t* codes[2];
@@ -84,8 +99,21 @@ struct Ctl {
   uint64_t full_a[kSlotsA], empty_a[kSlotsA], full_b[kSlotsB], empty_b[kSlotsB], acc_full, acc_empty;
   uint32_t tmem;
   int fail;   // a wait expired: the tile's outputs become NaN
-  int plain;  // batch rows (bits) to be summed by plain FMAs
+  uint32_t row_max[kRows];  // bits of the largest finite magnitude
+  uint32_t nan_rows, inf_rows;  // batch rows with a NaN, with an infinity (bits)
+  uint32_t infs;
+  int scan;  // a row of this block has an infinity or a NaN
+  int inf_row[kInfs], inf_at[kInfs];
 };
+
+__device__ __forceinline__ uint32_t mag(float f) { return __float_as_uint(f) & 0x7FFFFFFFu; }
+
+// The grid of a row whose largest magnitude has these bits: 2^k above it, k >= -126 (below, the
+// inputs are multiples of 2^-149, which the grid holds).
+__device__ __forceinline__ int grid_exp(uint32_t max_bits) { return (int)(max_bits >> 23) - 126; }
+__device__ __forceinline__ float exp2_bits(int e) {  // 2^e, -149 <= e <= 127
+  return __uint_as_float(e >= -126 ? (uint32_t)(e + 127) << 23 : 1u << (e + 149));
+}
 
 __device__ __forceinline__ bool ctl_wait(Ctl& c, uint64_t* bar, uint32_t parity) { return tc_wait(bar, parity, &c.fail); }
 
@@ -95,6 +123,56 @@ __device__ __forceinline__ uint2 plane_bytes(int p) {
          : p == 1 ? make_uint2(0x80000080u, 0x3F0000BFu)   // D_out: -1 0  0  1
          : p == 2 ? make_uint2(0x00808000u, 0x003F3F00u)   // E_in:  0  1  1  0
                   : make_uint2(0x80000080u, 0x3F00003Fu);  // E_out: 1  0  0  1
+}
+
+// inputs [n0, n0 + n) of a part of a matrix of length len
+struct Part {
+  int s0, stages;
+  __device__ Part(int64_t len, uint32_t part, uint32_t split) {
+    const uint32_t all = (uint32_t)((len + kStageK - 1) / kStageK);
+    s0 = (int)(all * part / split);
+    stages = (int)(all * (part + 1) / split) - s0;
+  }
+  __device__ int64_t n0() const { return (int64_t)kStageK * s0; }
+  __device__ int n(int64_t len) const {
+    return (int)(len - n0() < (int64_t)kStageK * stages ? len - n0() : (int64_t)kStageK * stages);
+  }
+};
+
+// The biased exponent of the largest magnitude of each row, plane and part (255: an infinity or
+// a NaN is among them), into byte 2 plane + part of the first output of every channel tile:
+// the tile's own CTAs read it before they write that output.  One CTA per row, plane and part.
+// With every tile taking the maxima of the same rows itself, 16 rows of the 7B layer took
+// 178 us (140 with this launch, which overlaps the tiles' set-up; 2 rows 126, now 121).
+__global__ void __launch_bounds__(kGridThreads) row_grid_kernel(const __grid_constant__ FoldTcParams p) {
+  __shared__ uint32_t wmax[kGridThreads / 32];
+  grid_dependents_start();  // the tiles' kernel sets itself up and waits for this one's end
+  const uint32_t split = (uint32_t)p.split, per = 2 * split * (uint32_t)p.rows;
+  const FoldTcMat& a = p.mat[blockIdx.x / per];
+  const uint32_t id = blockIdx.x % per;
+  const int64_t row = id / (2 * split);
+  const uint32_t pl = id / split % 2, part = id % split;
+  const Part range(a.n, part, split);
+  const int n = range.n(a.n);
+  const float* q = a.x[pl] + row * a.ldx + range.n0();
+  uint32_t m = 0u;
+  if (a.vec_x) {
+#pragma unroll 4
+    for (int i = 4 * threadIdx.x; i < n; i += 4 * kGridThreads) {
+      const float4 f = __ldg(reinterpret_cast<const float4*>(q + i));
+      m = max(m, max(max(mag(f.x), mag(f.y)), max(mag(f.z), mag(f.w))));
+    }
+  } else {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < n; i += kGridThreads) m = max(m, mag(__ldg(q + i)));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kGridThreads / 32; ++w) m = max(m, wmax[w]);
+  for (int64_t c = (int64_t)threadIdx.x * kTile; c < a.m; c += kGridThreads * kTile)
+    reinterpret_cast<uint8_t*>(a.y + row * a.ldy + c)[2 * pl + part] = (uint8_t)(m >> 23);
 }
 
 __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_constant__ FoldTcParams p) {
@@ -115,12 +193,11 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   const FoldTcMat& a = p.mat[mi];
   const int64_t c0 = (int64_t)(tile - p.tile0[mi]) * kTile;
   const int rows = p.rows - row0 < kRows ? p.rows - row0 : kRows;
-  const int nt = (3 * rows + 15) / 16 * 16;
+  const int nt = (kDigits * rows + 15) / 16 * 16;
   // this CTA's part of the inputs: n inputs from n0, in L stages (none where n < 64 split)
-  const uint32_t all = (uint32_t)((a.n + kStageK - 1) / kStageK);
-  const int s0 = (int)(all * part / split), L = (int)(all * (part + 1) / split) - s0;
-  const int64_t n0 = (int64_t)kStageK * s0;
-  const int n = (int)(a.n - n0 < (int64_t)kStageK * L ? a.n - n0 : (int64_t)kStageK * L);
+  const Part range(a.n, part, split);
+  const int s0 = range.s0, L = range.stages, n = range.n(a.n);
+  const int64_t n0 = range.n0();
 
   // decoding threads: channel r of the tile, its centres, its first code words
   const int grp = warp >> 2;
@@ -147,7 +224,6 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   uint4 w0 = fetch(grp), w1 = fetch(grp + 2), w2 = fetch(grp + 4);
   float4 cen = make_float4(0.f, 0.f, 0.f, 0.f);
   if (live) cen = __ldg(reinterpret_cast<const float4*>(a.centres[pl]) + c0 + r);
-  auto mag = [](float f) { return __float_as_uint(f) & 0x7FFFFFFFu; };
   const bool plain_channel = max(max(mag(cen.x), mag(cen.y)), max(mag(cen.z), mag(cen.w))) >= kBig;
 
   if (warp == kDecWarps + kSplitWarps) {
@@ -163,10 +239,86 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       mbar_init(&ctl.acc_full, 1);
       mbar_init(&ctl.acc_empty, kDecWarps);
       ctl.fail = 0;
-      ctl.plain = 0;
+      ctl.nan_rows = ctl.inf_rows = ctl.infs = 0u;
     }
+    // the exponents that row_grid_kernel left in the first word of the tile's output rows
+    uint32_t e = 0u;
+    grid_dependency_wait();
+    if (lane < rows)
+      e = reinterpret_cast<const volatile uint8_t*>(a.y + (int64_t)(row0 + lane) * a.ldy + c0)[2 * pl + part];
+    const bool scan = __any_sync(0xffffffffu, e == 255u);
+    if (lane < kRows) ctl.row_max[lane] = scan ? 0u : e << 23;
+    if (lane == 0) ctl.scan = scan;
     mbar_init_fence();
     tmem_alloc(&ctl.tmem, kCols);
+  }
+  __syncthreads();
+  // ---- rows with an infinity or a NaN: note them and take the others' largest magnitude
+  // (128 inputs of a row per warp and load) ----
+  if (ctl.scan) {
+    const float* x0 = a.x[pl] + (int64_t)row0 * a.ldx + n0;
+    const int blocks = (n + 127) / 128, tasks = rows * blocks;
+    const bool vec_x = a.vec_x;
+    constexpr int kStep = kThreads / 32;
+    const int drow = blocks ? kStep / blocks : 0, dblk = blocks ? kStep % blocks : 0;
+    int row = blocks ? warp / blocks : 0, blk = blocks ? warp % blocks : 0;
+    auto next = [&](int& r, int& b) {
+      r += drow;
+      b += dblk;
+      if (b >= blocks) {
+        b -= blocks;
+        ++r;
+      }
+    };
+    for (int t0 = warp; t0 < tasks; t0 += kScan * kStep) {
+      float4 f[kScan];
+      int lr = row, lb = blk;
+#pragma unroll
+      for (int k = 0; k < kScan; ++k) {
+        const int i = 128 * lb + 4 * lane;
+        const float* q = x0 + (int64_t)lr * a.ldx + i;
+        f[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lr < rows && i < n) {
+          if (vec_x) {
+            f[k] = __ldg(reinterpret_cast<const float4*>(q));
+          } else {
+            f[k].x = __ldg(q);
+            if (i + 1 < n) f[k].y = __ldg(q + 1);
+            if (i + 2 < n) f[k].z = __ldg(q + 2);
+            if (i + 3 < n) f[k].w = __ldg(q + 3);
+          }
+        }
+        next(lr, lb);
+      }
+#pragma unroll
+      for (int k = 0; k < kScan; ++k) {
+        if (row >= rows) break;
+        uint32_t m = max(max(mag(f[k].x), mag(f[k].y)), max(mag(f[k].z), mag(f[k].w)));
+        if (__any_sync(0xffffffffu, m >= kInf)) {
+          const float v[4] = {f[k].x, f[k].y, f[k].z, f[k].w};
+          m = 0u;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const uint32_t b = mag(v[e]);
+            if (b > kInf) {
+              atomicOr(&ctl.nan_rows, 1u << row);
+            } else if (b == kInf) {
+              atomicOr(&ctl.inf_rows, 1u << row);
+              const uint32_t at = atomicAdd(&ctl.infs, 1u);
+              if (at < (uint32_t)kInfs) {
+                ctl.inf_row[at] = row;
+                ctl.inf_at[at] = 128 * blk + 4 * lane + e;
+              }
+            } else {
+              m = max(m, b);
+            }
+          }
+        }
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) atomicMax(&ctl.row_max[row], m);
+        next(row, blk);
+      }
+    }
   }
   tc_fence_before();
   // centres symmetric about 0 in the whole tile: two planes suffice
@@ -221,7 +373,13 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
     const int seg = t & 7, br0 = t >> 3;
     const float* src = a.x[pl] + (int64_t)(row0 + br0) * a.ldx + n0 + 8 * seg;
     const bool vec_x = a.vec_x;
-    uint32_t big[2] = {0u, 0u};
+    float scale[2];  // 2^-k of the thread's rows
+    bool clean[2];   // all finite
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      scale[h] = exp2_bits(-grid_exp(ctl.row_max[br0 + 8 * h]));
+      clean[h] = (((ctl.nan_rows | ctl.inf_rows) >> (br0 + 8 * h)) & 1u) == 0u;
+    }
     auto load = [&](int st, float (&v)[2][8]) {
       const int i0 = kStageK * (st < L ? st : st - L);
       const int left = n - i0 - 8 * seg;
@@ -248,28 +406,33 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       for (int h = 0; h < 2; ++h) {
         const int br = br0 + 8 * h;
         if (br < rows) {
-          uint32_t pk[3][4];
+          uint32_t pk[kDigits][4];
+          const float2 sc = make_float2(scale[h], scale[h]);
+          auto digit = [](float2 t, float to) {  // nearest multiple of to's last place
+            return __fadd2_rn(__fadd2_rn(t, make_float2(to, to)), make_float2(-to, -to));
+          };
+          auto less = [](float2 t, float2 d) { return __fadd2_rn(t, make_float2(-d.x, -d.y)); };
+          auto pack = [](float2 d) { return prmt(__float_as_uint(d.x), __float_as_uint(d.y), 0x7632u); };
 #pragma unroll
-          for (int e = 0; e < 8; e += 2) {
+          for (int e = 0; e < 4; ++e) {
             // K order inside 8 inputs as the decoded codes': 0, 4, 1, 5, 2, 6, 3, 7
-            uint32_t b1[2], b2[2], b3[2];
-#pragma unroll
-            for (int o = 0; o < 2; ++o) {
-              const float x = v[h][e / 2 + 4 * o];
-              const uint32_t bits = __float_as_uint(x);
-              big[h] = max(big[h], bits & 0x7FFFFFFFu);
-              b1[o] = bits & 0xFFFF0000u;
-              const float rest = __fsub_rn(x, __uint_as_float(b1[o]));
-              b2[o] = __float_as_uint(rest) & 0xFFFF0000u;
-              b3[o] = __float_as_uint(__fsub_rn(rest, __uint_as_float(b2[o])));
+            float2 x = make_float2(v[h][e], v[h][e + 4]);
+            if (!clean[h]) {
+              if (mag(x.x) >= kInf) x.x = 0.f;
+              if (mag(x.y) >= kInf) x.y = 0.f;
             }
-            pk[0][e / 2] = prmt(b1[0], b1[1], 0x7632u);
-            pk[1][e / 2] = prmt(b2[0], b2[1], 0x7632u);
-            pk[2][e / 2] = prmt(b3[0], b3[1], 0x7632u);
+            const float2 t = __fmul2_rn(x, sc);
+            const float2 d1 = digit(t, 0x1.8p16f), t1 = less(t, d1);
+            const float2 d2 = digit(t1, 0x1.8p8f), t2 = less(t1, d2);
+            const float2 d3 = digit(t2, 0x1.8p0f), t3 = less(t2, d3);
+            pk[0][e] = pack(d1);
+            pk[1][e] = pack(d2);
+            pk[2][e] = pack(d3);
+            pk[3][e] = pack(t3);
           }
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            const uint32_t row = 3 * br + q;
+          for (int q = 0; q < kDigits; ++q) {
+            const uint32_t row = kDigits * br + q;
             sts128(ring + sb * kBBytes + row * 128 + ((seg ^ (row & 7)) << 4),
                    make_uint4(pk[q][0], pk[q][1], pk[q][2], pk[q][3]));
           }
@@ -289,9 +452,6 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       if (s + 2 < V) put(s + 2, vb);
       load(s + 6, vb);
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-      if (big[h] >= kBig) atomicOr(&ctl.plain, 1 << (br0 + 8 * h));
   } else {
     // ---- decode, and the fp32 sums ----
     const uint32_t lanes = tmem + ((uint32_t)(warp & 3) << 21);  // this warp's 32 TMEM lanes
@@ -313,20 +473,23 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
         fo = __fmul_rn(0.5f, e ? __fadd_rn(cen.w, cen.x) : __fsub_rn(cen.w, cen.x));
       }
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {  // four batch rows, twelve columns
+      for (int half = 0; half < 2; ++half) {  // four batch rows
         if (8 * grp + 4 * half < rows) {
-          float d[2][12];
+          float d[2][16];
 #pragma unroll
           for (int pn = 0; pn < 2; ++pn)
 #pragma unroll
-            for (int q = 0; q < 12; q += 4) tmem_ld4(&d[pn][q], lanes + pn * 64 + 24 * grp + 12 * half + q);
+            for (int q = 0; q < 16; q += 8) tmem_ld8(&d[pn][q], lanes + pn * 64 + 32 * grp + 16 * half + q);
           tmem_wait_ld();
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            // the three parts of the inputs, the smallest first
-            const float in = __fadd_rn(__fadd_rn(d[0][3 * k + 2], d[0][3 * k + 1]), d[0][3 * k]);
-            const float out = __fadd_rn(__fadd_rn(d[1][3 * k + 2], d[1][3 * k + 1]), d[1][3 * k]);
-            acc[4 * half + k] = __fadd_rn(acc[4 * half + k], __fmaf_rn(fo, out, __fmul_rn(fi, in)));
+            // the digits, the smallest first, then the row's 2^k (the rest beyond 2^100 at the end)
+            const float s2k = exp2_bits(min(grid_exp(ctl.row_max[8 * grp + 4 * half + k]), kTopExp));
+            float sum[2];
+#pragma unroll
+            for (int pn = 0; pn < 2; ++pn)
+              sum[pn] = __fmul_rn(__fadd_rn(__fadd_rn(__fadd_rn(d[pn][4 * k + 3], d[pn][4 * k + 2]), d[pn][4 * k + 1]), d[pn][4 * k]), s2k);
+            acc[4 * half + k] = __fadd_rn(acc[4 * half + k], __fmaf_rn(fo, sum[1], __fmul_rn(fi, sum[0])));
           }
         }
       }
@@ -370,24 +533,45 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   }
 
   __syncthreads();  // the MMAs have completed (their sums were waited for): shared memory is free
-  const int plain = *(volatile int*)&ctl.plain;
   const float bad = *(volatile int*)&ctl.fail ? __int_as_float(0x7FC00000) : 0.f;
   if (warp < kDecWarps) {
+    auto centre = [&](int i) {  // of input i
+      const uint32_t code = (__ldg(code_row + (i >> 4)) >> (2 * (i & 15))) & 3u;
+      return (code & 2u) ? ((code & 1u) ? cen.w : cen.z) : ((code & 1u) ? cen.y : cen.x);
+    };
+    const float* q = a.x[pl] + (int64_t)row0 * a.ldx + n0;
+    const uint32_t of = (0xFFu << (8 * grp)) & ((1u << rows) - 1u);  // this thread's rows
+    const bool many = ctl.infs > (uint32_t)kInfs;
+    const uint32_t infs = live && !many ? ctl.infs : 0u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const uint32_t row_max = ctl.row_max[8 * grp + k];
+      acc[k] = __fmul_rn(acc[k], exp2_bits(max(grid_exp(row_max) - kTopExp, 0)));
+    }
+    for (uint32_t e = 0; e < infs; ++e) {
+      const int row = ctl.inf_row[e], i = ctl.inf_at[e];
+      const float add = __fmul_rn(centre(i), __ldg(q + (int64_t)row * a.ldx + i));
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (row == 8 * grp + k) acc[k] = __fadd_rn(acc[k], add);
+    }
+    const uint32_t plain = of & (plain_channel ? ~0u : many ? ctl.inf_rows : 0u);
+    if (live && plain) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if ((plain >> (8 * grp + k)) & 1u) acc[k] = 0.f;
+      for (int i = 0; i < n; ++i) {
+        const float c = centre(i);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if ((plain >> (8 * grp + k)) & 1u) acc[k] = __fmaf_rn(c, __ldg(q + (int64_t)(8 * grp + k) * a.ldx + i), acc[k]);
+      }
+    }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int c = 8 * grp + k;
-      float v = acc[k];
-      if (c < rows && (plain_channel || ((plain >> c) & 1))) {
-        v = 0.f;
-        const float* q = a.x[pl] + (int64_t)(row0 + c) * a.ldx + n0;
-        const float cc[4] = {cen.x, cen.y, cen.z, cen.w};
-        for (int i = 0; live && i < n; ++i) {
-          const uint32_t code = (__ldg(code_row + (i >> 4)) >> (2 * (i & 15))) & 3u;
-          const float ce = (code & 2u) ? ((code & 1u) ? cc[3] : cc[2]) : ((code & 1u) ? cc[1] : cc[0]);
-          v = __fmaf_rn(ce, __ldg(q + i), v);
-        }
-      }
-      asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + r) * 4), "f"(__fadd_rn(v, bad)) : "memory");
+      const float nan = (ctl.nan_rows >> c) & 1u ? __int_as_float(0x7FC00000) : bad;
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + r) * 4), "f"(__fadd_rn(acc[k], nan)) : "memory");
     }
   }
   cluster_sync_all();
@@ -456,17 +640,21 @@ kd_status fold_tc_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStr
       tiles += (a.m + kTile - 1) / kTile;
     }
     if (tiles == 0) return KD_OK;
+    row_grid_kernel<<<(unsigned)(p.count * p.rows * 2 * p.split), kGridThreads, 0, s>>>(p);
+    if (cudaGetLastError() != cudaSuccess) return KD_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(tiles * p.row_blocks * 2 * p.split));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = (unsigned)(2 * p.split);
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     if (cudaLaunchKernelEx(&cfg, fold_tc_kernel, p) != cudaSuccess) return KD_ERR_CUDA;
   }
   return KD_OK;

@@ -135,6 +135,11 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* fai
   return false;
 }
 
+// Programmatic dependent launch: the next launch of the stream, if it asks for it, may start
+// once every CTA of this one has come here; it then waits for this one's end and its writes.
+__device__ __forceinline__ void grid_dependents_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));

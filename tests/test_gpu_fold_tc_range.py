@@ -1,0 +1,78 @@
+"""The fp32 product from the 2-bit planes on the tensor cores (two batch rows and more) over
+inputs whose magnitudes differ widely, against 64 bits from the same codes and centres.
+
+Tolerance, per row, of max |Y|: 1e-6, as in test_gpu_fold_tc.  The sums of the inputs' digits
+are exact to 2^-32 of the row's largest input each; after them come at most 12 fp32 roundings
+of values up to a few max |Y| (per plane and part three additions of the digits, two products
+and their sum; then the parts)."""
+
+import pytest
+import torch
+
+from tests.test_gpu_fold import kd  # noqa: F401  (the module's fixture)
+from tests.test_gpu_fold_tc import _case, _plane, _y64
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-6
+
+
+def _check(y, ref):
+    err = (y.double() - ref).abs().amax(1) / ref.abs().amax(1)
+    assert (err <= TOL).all(), err.max().item()
+
+
+@pytest.mark.parametrize("n,batch", [(256, 2), (768, 33), (4096, 16), (11008, 17)])
+@pytest.mark.parametrize("e", [10, 18, 26])
+def test_one_input_leads_the_row(kd, n, batch, e):  # noqa: F811
+    """One input 2^e times the others, at the first, the last or another place of the row."""
+    dec, x, xp = _case(kd, n, 130, batch)
+    for r in range(batch):
+        x[r, (0, n - 1, (37 * r) % n)[r % 3]] = 1.2345678 * 2.0 ** e
+    _check(kd.matmul_2bit(dec, x, xp), _y64(dec, x, xp))
+
+
+@pytest.mark.parametrize("n,batch", [(256, 33), (4096, 16), (11008, 5)])
+def test_log_normal_inputs(kd, n, batch):  # noqa: F811
+    dec, x, xp = _case(kd, n, 130, batch, kmeans=1)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    x *= torch.exp(2 * torch.randn(x.shape, generator=g, device="cuda"))
+    xp *= torch.exp(2 * torch.randn(x.shape, generator=g, device="cuda"))
+    _check(kd.matmul_2bit(dec, x, xp), _y64(dec, x, xp))
+
+
+@pytest.mark.parametrize("batch", [5, 20])
+@pytest.mark.parametrize("e", [-112, -120, -130, -140, 125])
+def test_rows_at_the_ends_of_the_range(kd, batch, e):  # noqa: F811
+    """Rows of 2^e, subnormal ones among them, beside an ordinary row; the centres are scaled
+    so that the results stay normal numbers."""
+    dec, x, xp = _case(kd, 1000, 130, batch)
+    dec.centres_u *= 2.0 ** (-40 if e > 0 else 40)
+    dec.centres_v *= 2.0 ** (-40 if e > 0 else 40)
+    x, xp = x.clamp(-4, 4), xp.clamp(-4, 4)
+    x[1:] *= 2.0 ** (e // 2)
+    xp[1:] *= 2.0 ** (e // 2)
+    x[1:] *= 2.0 ** (e - e // 2)
+    xp[1:] *= 2.0 ** (e - e // 2)
+    assert torch.isfinite(x).all() and (x[1:] != 0).any(1).all()
+    _check(kd.matmul_2bit(dec, x, xp), _y64(dec, x, xp))
+
+
+@pytest.mark.parametrize("count", [1, 2, 64, 65, 300])
+def test_infinities_of_a_row(kd, count):  # noqa: F811
+    """`count` infinities in one row: infinite where their products agree in sign, else NaN;
+    other rows keep their bits."""
+    n = 300
+    dec, x, xp = _case(kd, n, 140, 20)
+    ref = kd.matmul_2bit(dec, x, xp)
+    x2 = x.clone()
+    at = torch.arange(count, device="cuda") * 7 % n
+    x2[11, at] = float("inf")
+    y = kd.matmul_2bit(dec, x2, xp)
+    keep = [r for r in range(20) if r != 11]
+    assert torch.equal(y[keep], ref[keep])
+    sign = torch.sign(_plane(dec.codes_u, dec.centres_u, n)[:, at])
+    assert (sign != 0).all()
+    same = (sign == sign[:, :1]).all(1)
+    assert torch.equal(y[11][same], (sign[same, 0] * float("inf")).float())
+    assert torch.isnan(y[11][~same]).all()
