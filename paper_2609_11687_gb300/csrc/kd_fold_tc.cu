@@ -10,6 +10,8 @@
 //    multiply the inputs by planes of -1, 0 and 1, which are exact in bf16:
 //        D_in = T2 - T1, D_out = T3 - T0, and where a channel of the tile has centres that are
 //        not symmetric about 0 (after k-means refinement), E_in = T1 + T2, E_out = T0 + T3.
+//    A pair of centres far from symmetric takes T2 and T1 (T3 and T0) themselves instead: with
+//    D and E a centre's sum would come out of differences as large as the other centre's.
 //    The centres stay fp32 and multiply the sums.
 // The sums of d1, d2 and d3 are whole numbers of at most 24 bits for up to 2^17 inputs, so the
 // tensor core, which cuts each addition off instead of rounding it, adds them exactly; kChunk
@@ -117,12 +119,20 @@ __device__ __forceinline__ float exp2_bits(int e) {  // 2^e, -149 <= e <= 127
 
 __device__ __forceinline__ bool ctl_wait(Ctl& c, uint64_t* bar, uint32_t parity) { return tc_wait(bar, parity, &c.fail); }
 
-// code -> bf16 as (low bytes, high bytes) of codes 0..3
-__device__ __forceinline__ uint2 plane_bytes(int p) {
-  return p == 0   ? make_uint2(0x00808000u, 0x003FBF00u)   // D_in:  0 -1  1  0
-         : p == 1 ? make_uint2(0x80000080u, 0x3F0000BFu)   // D_out: -1 0  0  1
-         : p == 2 ? make_uint2(0x00808000u, 0x003F3F00u)   // E_in:  0  1  1  0
-                  : make_uint2(0x80000080u, 0x3F00003Fu);  // E_out: 1  0  0  1
+// Whether a pair of centres (low, high) is far from symmetric: each of its sums has its own
+// plane then.  Below this line the factors of D and E are within 1.67 of each other's centre.
+__device__ __forceinline__ bool far(float low, float high) {
+  return !(fabsf(__fadd_rn(low, high)) <= __fmul_rn(0.25f, __fsub_rn(high, low)));
+}
+
+// code -> bf16 as (low bytes, high bytes) of codes 0..3: the inner or the outer pair's plane of
+// the first or the second pass
+__device__ __forceinline__ uint2 plane_bytes(bool outer, bool second, bool own) {
+  const uint2 d = outer ? make_uint2(0x80000080u, 0x3F0000BFu)   // D_out: -1 0  0  1
+                        : make_uint2(0x00808000u, 0x003FBF00u);  // D_in:   0 -1 1  0
+  if (!own) return make_uint2(d.x, second ? d.y & 0x3F3F3F3Fu : d.y);  // E: the signs off
+  const uint32_t keep = outer ? (second ? 0x000000FFu : 0xFF000000u) : (second ? 0x0000FF00u : 0x00FF0000u);
+  return make_uint2(d.x & keep, d.y & keep & 0x3F3F3F3Fu);
 }
 
 // inputs [n0, n0 + n) of a part of a matrix of length len
@@ -325,6 +335,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   const int reps = __syncthreads_or(!(cen.x == -cen.w && cen.y == -cen.z)) ? 2 : 1;
   tc_fence_after();
   const uint32_t tmem = ctl.tmem;
+  const bool own_in = far(cen.y, cen.z), own_out = far(cen.x, cen.w);
   const int V = L * reps;  // stages of all passes
   // accumulations of one pass: kChunk stages each but the last
   const int chunks = (L + kChunk - 1) / kChunk;
@@ -465,12 +476,12 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       ctl_wait(ctl, &ctl.acc_full, done & 1);
       tc_fence_after();
       // factors of the inner and the outer plane: c2, c3 where the centres are symmetric,
-      // else half of c2 - c1, c3 - c0 for D and of c2 + c1, c3 + c0 for E
+      // else half of c2 - c1, c3 - c0 for D and of c2 + c1, c3 + c0 for E, or the centres
       float fi = cen.z, fo = cen.w;
       if (reps == 2) {
         const bool e = done >= chunks;
-        fi = __fmul_rn(0.5f, e ? __fadd_rn(cen.z, cen.y) : __fsub_rn(cen.z, cen.y));
-        fo = __fmul_rn(0.5f, e ? __fadd_rn(cen.w, cen.x) : __fsub_rn(cen.w, cen.x));
+        fi = own_in ? (e ? cen.y : cen.z) : __fmul_rn(0.5f, __fadd_rn(cen.z, e ? cen.y : -cen.y));
+        fo = own_out ? (e ? cen.x : cen.w) : __fmul_rn(0.5f, __fadd_rn(cen.w, e ? cen.x : -cen.x));
       }
 #pragma unroll
       for (int half = 0; half < 2; ++half) {  // four batch rows
@@ -500,14 +511,17 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       next_end();
     };
     // own stages grp, grp + 2, ..., their code words loaded three own stages ahead
+    uint2 b0 = plane_bytes(false, false, own_in), b1 = plane_bytes(true, false, own_out);
 #pragma unroll 1
     for (int i = grp; i < V; i += 2) {
       const uint32_t ww[4] = {w0.x, w0.y, w0.z, w0.w};
       w0 = w1;
       w1 = w2;
       w2 = fetch(i + 6);
-      const bool e = i >= L;
-      const uint2 b0 = plane_bytes(e ? 2 : 0), b1 = plane_bytes(e ? 3 : 1);
+      if (i >= L && i < L + 2) {  // the first one of the second pass
+        b0 = plane_bytes(false, true, own_in);
+        b1 = plane_bytes(true, true, own_out);
+      }
       if (i >= kSlotsA) ctl_wait(ctl, &ctl.empty_a[grp], (i / kSlotsA - 1) & 1);
       tc_fence_after();  // the MMAs that read the slot are complete
 #pragma unroll
