@@ -373,11 +373,14 @@ kd_status kd_measure_fp32_peak(double* tflops, void* stream);
  *   xp                 device fp32, the same rows times P (kd_apply_p with the matrix's
  *                      sign seed on the rows of X), same layout and ldx.
  *   y                  device fp32, batch rows of m outputs, row r at y + r*ldy (ldy >= m).
- * Every code word is read once per group of up to 16 batch rows; the sums run in a fixed
- * order that depends on the batch size (deterministic).  With two rows and more an input is
- * taken to 2^-32 of the largest magnitude of its row (or of either half of the row) and the
- * sums of the inputs of one code are exact; every other operation is fp32.  y holds scratch
- * values until the call's last kernel has written it, and must not overlap the inputs.  A wait
+ * One of two kernels runs, by n, m and batch.  Few rows (one, mostly two, up to 16 of long
+ * vectors with few channels) look the centres up and sum in fp32, each row the same bits
+ * whatever the batch, every code word read once per two rows.  The others run on the tensor
+ * cores, every code word read once per 16 rows: an input is taken to 2^-32 of the largest
+ * magnitude of its row (or of either half of the row), the sums of the inputs of one code are
+ * exact, every other operation is fp32.  The order of the sums is fixed (deterministic) and
+ * depends on the batch.  y holds scratch values until the call's last kernel has written it,
+ * and must not overlap the inputs.  A wait
  * inside the kernel that exceeds its time limit leaves NaN in the outputs it concerns.  Errors: KD_ERR_INVALID_ARG (sizes, null or
  * unaligned pointers when m > 0 and batch > 0), KD_ERR_CUDA (launch).  m == 0 or
  * batch == 0 enqueues nothing. */
@@ -385,8 +388,8 @@ kd_status kd_matmul_2bit(const uint32_t* codes_u, const uint32_t* codes_v, const
                          const float* centres_v, int64_t n, int64_t m, const float* x, const float* xp,
                          int64_t batch, int64_t ldx, float* y, int64_t ldy, void* stream);
 
-/* kd_matmul_2bit for several matrices in one launch (a layer's products for one batch
- * of activations): each descriptor as kd_matmul_2bit's arguments, each matrix with its
+/* kd_matmul_2bit for several matrices, those of one kernel in one launch (a layer's products
+ * for one batch of activations): each descriptor as kd_matmul_2bit's arguments, each matrix with its
  * own n, m, inputs and output.  mats is a HOST array of 1 <= count <= KD_MAX_BATCH
  * descriptors read during the call.  Results equal kd_matmul_2bit's per matrix, bit for
  * bit.  Errors as kd_matmul_2bit (the first invalid matrix's), and KD_ERR_INVALID_ARG

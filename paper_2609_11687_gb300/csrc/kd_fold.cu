@@ -7,20 +7,21 @@
 // with xp = X P from kd_apply_p.  Neither U_q nor V_q is expanded: every weight costs
 // its 2-bit code in each plane (0.5 byte per weight in all), read once from HBM.
 //
-// This file holds the argument checks, the entry points and the kernel for one batch row;
-// two rows and more take kd_fold_tc.cu, on the tensor cores, 16 rows in one pass over the
-// codes (7B layer: 116 us at 2 rows and 131 at 16, where this kernel, two rows at a time,
-// took 121 and 970; at one row it takes 85).
+// This file holds the argument checks, the entry points and the table-lookup kernel for few
+// batch rows; the others take kd_fold_tc.cu, on the tensor cores, 16 rows in one pass over the
+// codes (by_lookup has the line and both sides' times).
 //
 // Mapping.  One launch serves up to KD_MAX_BATCH matrices (a layer): persistent CTAs
-// of eight warps walk the work items (matrix, tile of RT = 16 output channels).
+// of eight warps walk the work items (matrix, tile of RT = 16 / B output channels), for B
+// batch rows (blockIdx.y).
 // Per item each warp takes slices of 32 consecutive code words (512 inputs): it loads
 // its lane's 16 inputs of x and xp (L2-resident, shared by every item of the matrix)
 // into registers, then the code words of all RT channels of the tile (one coalesced
 // word per channel, plane and lane, all in flight together).  Two codes at a time (4
 // bits) index a per-channel table of the 16 centre pairs (c[q0], c[q1]) in shared
-// memory: one 64-bit shared load and one packed FP32x2 FMA per two weights and plane.  The lanes' and warps' partial sums are added in a fixed order
-// (deterministic results).
+// memory: one 64-bit shared load and one packed FP32x2 FMA per two weights, plane
+// and batch row.  The lanes' and warps' partial sums are added in a fixed order
+// (deterministic results, the same for one row and for two).
 #include <cuda_runtime.h>
 
 #include "kashin.h"
@@ -40,26 +41,38 @@ struct FoldMat {
   const float* x;
   const float* xp;
   float* y;
-  int64_t n, m, words;
+  int64_t n, m, words, ldx, ldy;
   int64_t tile0;  // first work item of this matrix
-  int vec;        // x and xp 16-byte aligned: 128-bit input loads
+  int vec;        // x and xp 16-byte aligned with ldx a multiple of 4: 128-bit input loads
 };
 
 struct FoldParams {
   int count;
-  int64_t items;   // work items of all matrices
+  int rows;        // batch rows of the call
+  int64_t items;   // work items of all matrices, once for each B rows (blockIdx.y)
   FoldMat mat[KD_MAX_BATCH];
 };
 
-constexpr int RT = 16;  // output channels per work item: partial sums per lane
+// RT x B = 16 partial sums per lane
+template <int B>
+struct FoldTile {
+  static constexpr int RT = 16 / B;
+};
 
+// MANY: more than B batch rows (without, the row offsets fold away: 7B layer, two rows, 131 ->
+// 125 us)
+template <int B, bool MANY>
 __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_constant__ FoldParams p) {
+  constexpr int RT = FoldTile<B>::RT;
+  constexpr int K = RT * B;  // partial sums per lane
+  static_assert(K == 16, "the reduction scatters 16 values per lane");
   __shared__ float2 tab[2 * RT * 16];
   __shared__ float red[kFoldWarps * 16];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
 
   int mi = 0;
+  const int row0 = MANY ? B * blockIdx.y : 0;
   for (int64_t item = blockIdx.x; item < p.items; item += gridDim.x) {
     while (mi + 1 < p.count && item >= p.mat[mi + 1].tile0) ++mi;
     const FoldMat& a = p.mat[mi];
@@ -80,9 +93,11 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
     }
     __syncthreads();
 
-    float2 acc[RT];
+    float2 acc[RT][B];
 #pragma unroll
-    for (int r = 0; r < RT; ++r) acc[r] = make_float2(0.f, 0.f);
+    for (int r = 0; r < RT; ++r)
+#pragma unroll
+      for (int b = 0; b < B; ++b) acc[r][b] = make_float2(0.f, 0.f);
 
     const int64_t nslices = (a.words + 31) / 32;
     for (int64_t s = warp; s < nslices; s += kFoldWarps) {
@@ -95,26 +110,34 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
         cu[r] = ok ? __ldg(a.codes_u + (j0 + r) * a.words + wi) : 0u;
         cv[r] = ok ? __ldg(a.codes_v + (j0 + r) * a.words + wi) : 0u;
       }
-      // this lane's 16 inputs of x and xp (zero past n): four 128-bit loads each when the
-      // whole word lies inside aligned rows
-      float2 xv[8], pv[8];
-      if (valid && a.vec && 16 * wi + 16 <= a.n) {
+      // this lane's 16 inputs of x and xp per batch row (zero past n and past the rows):
+      // four 128-bit loads each when the whole word lies inside aligned rows
+      float2 xv[B][8], pv[B][8];
+      {
+        const bool vec = a.vec && 16 * wi + 16 <= a.n;
 #pragma unroll
-        for (int k = 0; k < 8; k += 2) {
-          const float4 u = __ldg(reinterpret_cast<const float4*>(a.x + 16 * wi + 2 * k));
-          const float4 w = __ldg(reinterpret_cast<const float4*>(a.xp + 16 * wi + 2 * k));
-          xv[k] = make_float2(u.x, u.y);
-          xv[k + 1] = make_float2(u.z, u.w);
-          pv[k] = make_float2(w.x, w.y);
-          pv[k + 1] = make_float2(w.z, w.w);
-        }
-      } else {
+        for (int b = 0; b < B; ++b) {
+          const bool live = valid && row0 + b < p.rows;
+          const int64_t o0 = (int64_t)(row0 + b) * a.ldx + 16 * wi;
+          if (vec && live) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const int64_t i = 16 * wi + 2 * k;
-          const bool i0 = valid && i < a.n, i1 = valid && i + 1 < a.n;
-          xv[k] = make_float2(i0 ? __ldg(a.x + i) : 0.f, i1 ? __ldg(a.x + i + 1) : 0.f);
-          pv[k] = make_float2(i0 ? __ldg(a.xp + i) : 0.f, i1 ? __ldg(a.xp + i + 1) : 0.f);
+            for (int k = 0; k < 8; k += 2) {
+              const float4 u = __ldg(reinterpret_cast<const float4*>(a.x + o0 + 2 * k));
+              const float4 w = __ldg(reinterpret_cast<const float4*>(a.xp + o0 + 2 * k));
+              xv[b][k] = make_float2(u.x, u.y);
+              xv[b][k + 1] = make_float2(u.z, u.w);
+              pv[b][k] = make_float2(w.x, w.y);
+              pv[b][k + 1] = make_float2(w.z, w.w);
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int64_t i = 16 * wi + 2 * k;
+              const bool i0 = live && i < a.n, i1 = live && i + 1 < a.n;
+              xv[b][k] = make_float2(i0 ? __ldg(a.x + o0 + 2 * k) : 0.f, i1 ? __ldg(a.x + o0 + 2 * k + 1) : 0.f);
+              pv[b][k] = make_float2(i0 ? __ldg(a.xp + o0 + 2 * k) : 0.f, i1 ? __ldg(a.xp + o0 + 2 * k + 1) : 0.f);
+            }
+          }
         }
       }
 #pragma unroll
@@ -123,19 +146,24 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
         for (int k = 0; k < 8; ++k) {
           const float2 tu = tab[r * 16 + ((cu[r] >> (4 * k)) & 15u)];
           const float2 tv = tab[(RT + r) * 16 + ((cv[r] >> (4 * k)) & 15u)];
-          acc[r] = __ffma2_rn(tu, xv[k], acc[r]);
-          acc[r] = __ffma2_rn(tv, pv[k], acc[r]);
+#pragma unroll
+          for (int b = 0; b < B; ++b) {
+            acc[r][b] = __ffma2_rn(tu, xv[b][k], acc[r][b]);
+            acc[r][b] = __ffma2_rn(tv, pv[b][k], acc[r][b]);
+          }
         }
       }
     }
 
     // lane sums, then a butterfly reduce-scatter: lane l ends with its warp's total of
-    // channel l % 16
-    float v[RT];
+    // value l % 16 (value index r * B + b)
+    float v[K];
 #pragma unroll
-    for (int r = 0; r < RT; ++r) v[r] = __fadd_rn(acc[r].x, acc[r].y);
+    for (int r = 0; r < RT; ++r)
 #pragma unroll
-    for (int k = RT / 2; k >= 1; k >>= 1) {
+      for (int b = 0; b < B; ++b) v[r * B + b] = __fadd_rn(acc[r][b].x, acc[r][b].y);
+#pragma unroll
+    for (int k = K / 2; k >= 1; k >>= 1) {
 #pragma unroll
       for (int i = 0; i < k; ++i) {
         const bool hi = (lane & k) != 0;
@@ -145,27 +173,29 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
       }
     }
     v[0] = __fadd_rn(v[0], __shfl_xor_sync(0xffffffffu, v[0], 16));
-    if (lane < RT) red[warp * 16 + lane] = v[0];
+    if (lane < K) red[warp * 16 + lane] = v[0];
     __syncthreads();
-    if (threadIdx.x < RT) {
+    if (threadIdx.x < K) {
       float t = red[threadIdx.x];
 #pragma unroll
       for (int w = 1; w < kFoldWarps; ++w) t = __fadd_rn(t, red[w * 16 + threadIdx.x]);
-      if (j0 + threadIdx.x < a.m) a.y[j0 + threadIdx.x] = t;
+      const int r = threadIdx.x / B, b = threadIdx.x % B;
+      if (j0 + r < a.m && row0 + b < p.rows) a.y[(int64_t)(row0 + b) * a.ldy + j0 + r] = t;
     }
   }
 }
 
+template <int B, bool MANY>
 cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
   int dev = 0, sms = 0, per = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fold_kernel, kFoldThreads, 0)) != cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fold_kernel<B, MANY>, kFoldThreads, 0)) != cudaSuccess)
     return e;
   if (per < 1) return cudaErrorInvalidConfiguration;
   const int64_t grid = p.items < (int64_t)per * sms ? p.items : (int64_t)per * sms;
-  fold_kernel<<<(unsigned)grid, kFoldThreads, 0, s>>>(p);
+  fold_kernel<B, MANY><<<dim3((unsigned)grid, (unsigned)((p.rows + B - 1) / B)), kFoldThreads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -190,21 +220,20 @@ kd_status check_fold(const kd_fold_mat& a, int64_t batch) {
 }  // namespace
 }  // namespace kd
 
-extern "C" kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, int64_t batch, void* stream) {
-  if (!mats || count < 1 || count > KD_MAX_BATCH || batch < 0) return KD_ERR_INVALID_ARG;
-  for (int i = 0; i < count; ++i) {
-    const kd_status st = kd::check_fold(mats[i], batch);
-    if (st != KD_OK) return st;
-  }
-  if (batch == 0) return KD_OK;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (batch > 1) return kd::fold_tc_run(mats, count, batch, s);
-  kd::FoldParams p;
-  p.count = count;
-  int64_t items = 0;
+namespace kd {
+namespace {
+
+template <int B>
+kd_status fold_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStream_t s) {
+  constexpr int RT = FoldTile<B>::RT;
+  FoldParams p;
+  p.count = 0;
+  p.rows = (int)batch;
+  p.items = 0;
   for (int i = 0; i < count; ++i) {
     const kd_fold_mat& a = mats[i];
-    kd::FoldMat& f = p.mat[i];
+    if (a.m == 0) continue;
+    FoldMat& f = p.mat[p.count++];
     f.codes_u = a.codes_u;
     f.codes_v = a.codes_v;
     f.centres_u = a.centres_u;
@@ -215,13 +244,64 @@ extern "C" kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, in
     f.n = a.n;
     f.m = a.m;
     f.words = (a.n + 15) / 16;
-    f.tile0 = items;
-    f.vec = kd::aligned(f.x, 16) && kd::aligned(f.xp, 16);
-    items += (a.m + kd::RT - 1) / kd::RT;
+    f.ldx = a.ldx;
+    f.ldy = a.ldy;
+    f.tile0 = p.items;
+    f.vec = aligned(f.x, 16) && aligned(f.xp, 16) && (a.ldx % 4 == 0 || batch == 1);
+    p.items += (a.m + RT - 1) / RT;
   }
-  p.items = items;
-  if (items > 0 && kd::launch_fold(p, s) != cudaSuccess) return KD_ERR_CUDA;
-  return KD_OK;
+  if (p.items == 0) return KD_OK;
+  const cudaError_t e = batch > B ? launch_fold<B, (B > 1)>(p, s) : launch_fold<B, false>(p, s);
+  return e == cudaSuccess ? KD_OK : KD_ERR_CUDA;
+}
+
+}  // namespace
+}  // namespace kd
+
+namespace kd {
+namespace {
+
+// Whether a matrix takes the lookup kernel.  It re-reads the codes for every two rows but has
+// a short chain per item; the tensor-core kernel has the same time up to 16 rows and up to about
+// 9000 channels, 11 us at n = 256, 13 at 768, 17 at 2048, 23 at 4096, 44 at 11008 (nearly twice
+// that with centres that are not symmetric).  Measured, lookup against tensor cores (us):
+//   one row     always (7B layer 86)
+//   two rows    4096 x 300 11 / 23, 4096 x 4096 19 / 23, 4096 x 11008 35 / 43, 7B layer 125 / 123
+//               (125 / 217 not symmetric), 768 x 768 10 / 13; short vectors of many channels the
+//               other way: 768 x 4096 15 / 13, 256 x 11008 26 / 17
+//   3, 4 rows   4096 x 300 9 / 23, 4096 x 2048 18 / 23, 4096 x 3072 24 / 23, 11008 x 2048 36 / 44
+//   8, 16 rows  4096 x 1024 18 / 23, 27 / 23; 16384 x 300 18 / 59, 26 / 64
+// Below n = 4096 three rows and more stay with the tensor cores although single matrices would
+// gain up to 8 us (3072 x 768 13 / 19): the layers of such models are called whole, and two
+// launches cost them more (768-wide layer, 4 rows: 21 us in one).  By the matrix and the batch
+// alone, so that a matrix gives the same bits alone and in a batched call.
+bool by_lookup(const kd_fold_mat& a, int64_t batch) {
+  if (batch == 1) return true;
+  if (batch == 2) return a.n >= 1024 || a.m <= 3072;
+  return batch <= 16 && a.n >= 4096 && a.m <= 4096 && a.m * ((batch + 1) / 2) <= 4096;
+}
+
+}  // namespace
+}  // namespace kd
+
+extern "C" kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, int64_t batch, void* stream) {
+  if (!mats || count < 1 || count > KD_MAX_BATCH || batch < 0) return KD_ERR_INVALID_ARG;
+  for (int i = 0; i < count; ++i) {
+    const kd_status st = kd::check_fold(mats[i], batch);
+    if (st != KD_OK) return st;
+  }
+  if (batch == 0) return KD_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  kd_fold_mat sorted[KD_MAX_BATCH];
+  int few = 0, rest = 0;
+  for (int i = 0; i < count; ++i)
+    if (kd::by_lookup(mats[i], batch)) sorted[few++] = mats[i];
+  for (int i = 0; i < count; ++i)
+    if (!kd::by_lookup(mats[i], batch)) sorted[few + rest++] = mats[i];
+  kd_status st = KD_OK;
+  if (few) st = batch == 1 ? kd::fold_run<1>(sorted, few, batch, s) : kd::fold_run<2>(sorted, few, batch, s);
+  if (st == KD_OK && rest) st = kd::fold_tc_run(sorted + few, rest, batch, s);
+  return st;
 }
 
 extern "C" kd_status kd_matmul_2bit(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,

@@ -76,3 +76,16 @@ def test_infinities_of_a_row(kd, count):  # noqa: F811
     same = (sign == sign[:, :1]).all(1)
     assert torch.equal(y[11][same], (sign[same, 0] * float("inf")).float())
     assert torch.isnan(y[11][~same]).all()
+
+
+def test_vectors_beyond_one_accumulation(kd):  # noqa: F811
+    """2^16 inputs fill an accumulation: one stage into a second one, all inputs of one sign."""
+    n, m, batch = 65600, 129, 17
+    g = torch.Generator(device="cuda").manual_seed(1)
+    codes = [torch.randint(-2 ** 31, 2 ** 31, (m, n // 16), generator=g, device="cuda").int() for _ in range(2)]
+    c = torch.tensor([-1.5, -0.4, 0.4, 1.5], device="cuda").repeat(m, 1)
+    dec = kd.Decomposed(*codes, c, c.clone(), None, None, None, None, None)
+    x = torch.rand((batch, n), generator=g, device="cuda") + 1.0
+    xp = torch.rand((batch, n), generator=g, device="cuda") + 1.0
+    ref = torch.cat([_y64(dec, x[r:r + 1], xp[r:r + 1]) for r in range(batch)])
+    _check(kd.matmul_2bit(dec, x, xp), ref)
