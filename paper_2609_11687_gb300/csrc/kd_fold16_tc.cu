@@ -15,10 +15,11 @@
 //    fill them instead, element by element;
 //  * one thread issues the MMAs.
 // The accumulators live in TMEM, in two buffers where they fit beside the A slots (up to 128
-// rows).  Every kChunk units the decoding warps add the finished sums to fp32 registers,
-// while the next ones go to the other buffer: the tensor core adds with less than fp32's
-// rounding, so its chains are kept at 64 steps (half of what a warp of the mma.sync kernel
-// had at n = 4096).
+// rows).  Every few units the decoding warps add the finished sums to fp32 registers,
+// while the next ones go to the other buffer: the tensor core cuts its additions off instead of
+// rounding them, so its chains are kept at n / 32 steps (those of the mma.sync kernel's four
+// warps), between 8 and 64.  With 64 at every n, the error at n = 768 and more than 128 rows was
+// 1.1e-6 of the result's norm (2.2 times the mma.sync kernel's), at n = 256 3.5 times.
 //
 // Split of K.  The decode of 128 x 128 weights costs 370 SM cycles of the ALU pipe at least,
 // the MMAs 4 N, so up to about 90 rows the time is the decode's and every SM has to take its
@@ -44,7 +45,7 @@ namespace {
 constexpr int kTile = 128;        // output channels per CTA (the MMA's M, the TMEM lanes)
 constexpr int kStageK = 64;       // inputs per stage: one 128-byte row of 16-bit values
 constexpr int kUnitK = 128;       // inputs per unit: two stages
-constexpr int kChunk = 8;         // units per TMEM accumulation (64 MMA steps)
+constexpr int kChunk = 8;         // units per TMEM accumulation at most (64 MMA steps)
 constexpr int kDecWarps = 16;     // decoding warps: two groups of eight
 constexpr int kThreads = 32 * (kDecWarps + 2);  // + the TMA warp and the MMA warp
 constexpr int kMaxA = 4;          // A slots (units), at most
@@ -62,6 +63,7 @@ struct alignas(128) FoldTcMat {
   float* y;
   int64_t n, m, words, ldx, ldy;
   int units;       // units of one plane
+  int chunk;       // units per TMEM accumulation
   int vec;        // code rows 16-byte aligned: 128-bit code loads
 };
 
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
   while (mi + 1 < p.count && tile >= p.tile0[mi + 1]) ++mi;
   const FoldTcMat& a = p.mat[mi];
   const int64_t c0 = (int64_t)(tile - p.tile0[mi]) * kTile;
-  const int ku = a.units;
+  const int ku = a.units, chunk = a.chunk;
   const int k0 = (int)((uint32_t)(2 * ku) * rank / split);
   const int L = (int)((uint32_t)(2 * ku) * (rank + 1) / split) - k0;
 
@@ -224,11 +226,11 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
     // ---- MMAs ----
     const uint32_t idesc = tc_idesc(BF, nt);
     const uint64_t db0 = tc_desc(ring);
-    int s = 0, sa = 0, left = kChunk;  // units left of this accumulation
+    int s = 0, sa = 0, left = chunk;  // units left of this accumulation
     uint32_t par = 0, par_a = 0, b = 0, par_acc = 1;
     bool ok = true, fresh = true;
     for (int u = 0; u < L && ok; ++u) {
-      if (u >= NB * kChunk && fresh) ok = ctl_wait(&ctl, &ctl.acc_empty[b], par_acc);
+      if (u >= NB * chunk && fresh) ok = ctl_wait(&ctl, &ctl.acc_empty[b], par_acc);
       ok = ok && ctl_wait(&ctl, &ctl.full_a[sa], par_a);
       const uint32_t ta = tmem + NB * NTC + sa * kACols;
       const uint32_t d = tmem + b * NTC;
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
       }
       fresh = --left == 0;
       if (fresh) {
-        left = kChunk;
+        left = chunk;
         if (NB == 2) b ^= 1;
         if (b == 0) par_acc ^= 1;
       }
@@ -332,10 +334,11 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl.full_a[s]);
       // past the end of an accumulation (with two buffers, when its MMAs are known to be
-      // complete): they need nothing more from this warp
-      if (u >= (done + 1) * kChunk + (NB == 2 ? SA - 1 : 0)) promote();
+      // complete): they need nothing more from this warp.  All that ended: an accumulation may be
+      // one unit, and own units are two apart
+      while (u >= (done + 1) * chunk + (NB == 2 ? SA - 1 : 0)) promote();
     }
-    const int chunks = (L + kChunk - 1) / kChunk;
+    const int chunks = (L + chunk - 1) / chunk;
     while (done < chunks) promote();
   }
 
@@ -499,6 +502,7 @@ kd_status fold16_tc_run(const kd_fold_mat_f16* mats, int count, int64_t batch, c
         f.ldy = a.ldy;
         p.tile0[p.count] = (uint32_t)tiles;
         f.units = (int)((a.n + kUnitK - 1) / kUnitK);
+        f.chunk = a.n < 512 ? 1 : a.n / 256 < kChunk ? (int)(a.n / 256) : kChunk;
         f.vec = aligned_to(a.codes_u, 16) && aligned_to(a.codes_v, 16) && f.words % 4 == 0;
         if (tma && (!encode_rows(&f.map_x, f.x, a.n, p.rows, a.ldx, p.nt) ||
                     !encode_rows(&f.map_xp, f.xp, a.n, p.rows, a.ldx, p.nt)))
