@@ -423,8 +423,8 @@ kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, int64_t batch
  *           2-byte aligned; 16-byte aligned rows (base and ldx a multiple of 8) take
  *           128-bit loads.
  * The centres must be finite in fp16 (|c| <= 65504): a code padding past n multiplies
- * a zero input by a centre.  Every code word is read once per block of up
- * to 256 batch rows; the sums run in a fixed order that depends on
+ * a zero input by a centre.  Every code word is read once per block of up to 256 batch rows (16
+ * for short vectors of many channels); the sums run in a fixed order that depends on n, m and
  * the batch size (deterministic).  A wait inside the kernel that exceeds its time limit
  * leaves NaN in the outputs it concerns.  Errors and empty calls as kd_matmul_2bit. */
 kd_status kd_matmul_2bit_f16(const uint32_t* codes_u, const uint32_t* codes_v, const float* centres_u,
@@ -432,7 +432,7 @@ kd_status kd_matmul_2bit_f16(const uint32_t* codes_u, const uint32_t* codes_v, c
                              int64_t batch, int64_t ldx, float* y, int64_t ldy, void* stream);
 
 /* kd_matmul_2bit_f16 for several matrices in one launch (one more for matrices whose rows
- * are not 16-byte aligned); each descriptor as kd_matmul_2bit_f16's arguments.  mats is a
+ * are not 16-byte aligned, and one for short vectors of many channels); each descriptor as kd_matmul_2bit_f16's arguments.  mats is a
  * HOST array of 1 <= count <= KD_MAX_BATCH descriptors.  Results equal kd_matmul_2bit_f16's per matrix, bit for bit.
  * Errors as kd_matmul_2bit_batch. */
 typedef struct kd_fold_mat_f16 {

@@ -5,16 +5,15 @@
 //
 // with x, xp in the 16-bit type (xp = X P from kd_apply_p, rounded by the caller), h()
 // the rounding of a centre to that type, fp32 accumulation.  Neither plane is expanded
-// in memory.  This file holds the kernel for up to 8 batch rows (decode), the argument
-// checks and the entry points; more rows take kd_fold16_tc.cu, whose tcgen05 form decodes
-// every code once per 256 rows (7B layer: 84 us at 9 to 17 rows and 286 us at 512, where 16
-// rows at a time through mma.sync took 100 us and 3.2 ms; at 8 rows and fewer it is the
-// slower one, 83 against 78 us).
+// in memory.  This file holds the mma.sync kernel for few batch rows, the argument checks and
+// the entry points; the others take kd_fold16_tc.cu, whose tcgen05 form decodes every code once
+// per 256 rows (7B layer: 86 us at 9 rows and 286 us at 512, where 16 rows at a time through
+// mma.sync took 100 us and 3.2 ms; at 8 rows and fewer it is the slower one, 83 against 80 us).
 //
-// Mapping.  mma.m16n8k16 with M = the batch rows (the upper eight unused), N = 8 output
-// channels, K = 16 inputs: each code becomes its 16-bit centre in registers (kd_dec16.cuh)
-// and feeds a B fragment directly.  A work item is a tile of 32 channels (four n-tiles) of
-// one matrix and one CTA; its warps split the inputs into groups of 64 (four k-steps)
+// Mapping.  mma.m16n8k16 with M = the batch rows (the upper eight only in the form for more than
+// 8 rows), N = 8 output channels, K = 16 inputs: each code becomes its 16-bit centre in registers
+// (kd_dec16.cuh) and feeds a B fragment directly.  A work item is a tile of 32 channels (four
+// n-tiles) of one matrix and one CTA; its warps split the inputs into groups of 64 (four k-steps)
 // round-robin, each loading the next group's code words and inputs while it computes the
 // current one, then add their partial tiles in a fixed order (deterministic results).  Items
 // are numbered longest vectors first, so the hardware starts the long ones first.  Bound by
@@ -36,11 +35,12 @@
 namespace kd {
 namespace {
 
-// Warps of a CTA, which split the inputs: eight (two CTAs per SM).  With four, the last items
-// of a 7B layer ran on a third of the SMs: 86 us per layer at 4 rows, 78 with eight.
-constexpr int W = 8;
-constexpr int kF16Threads = 32 * W;
-constexpr int kF16Rows = 8;   // batch rows at most
+// Warps of a CTA, which split the inputs: eight (two CTAs per SM), with four the last items
+// of a 7B layer ran on a third of the SMs (86 us per layer at 4 rows, 80 with eight).  Short
+// vectors of many channels (wide_short) have four: eight would have one or two groups each and
+// spend their time around them (50257 x 768 at 8 rows: 31 us, 25 with four).
+constexpr int kF16Warps = 8, kF16ShortWarps = 4;
+constexpr int kF16Rows = 8;   // batch rows at most, 16 with the upper ones
 constexpr int kF16Tile = 32;  // output channels per work item (four n-tiles)
 constexpr int kRedStride = kF16Tile + 1;
 
@@ -59,7 +59,7 @@ struct Fold16Mat {
 
 struct Fold16Params {
   int count;
-  int rows;  // batch rows (<= 8)
+  int rows;  // batch rows of the call
   int64_t items;
   DecodeMul mul;
   Fold16Mat mat[KD_MAX_BATCH];
@@ -105,9 +105,13 @@ __device__ __forceinline__ void load_row16(uint32_t (&r)[8], const unsigned shor
   }
 }
 
-template <bool BF>
-__global__ void __launch_bounds__(kF16Threads, 2) fold16_kernel(const __grid_constant__ Fold16Params p) {
-  __shared__ float red[W][kF16Rows][kRedStride];
+// HI: 16 batch rows (blockIdx.y counts blocks of them), else up to 8; W: warps per work item
+template <bool BF, bool HI, int W>
+__global__ void __launch_bounds__(32 * W, W == kF16Warps ? 2 : HI ? 3 : 4)
+    fold16_kernel(const __grid_constant__ Fold16Params p) {
+  constexpr int kThreads = 32 * W, kRows = HI ? 2 * kF16Rows : kF16Rows;
+  __shared__ float red[W][kRows][kRedStride];
+  const int row0 = HI ? kRows * blockIdx.y : 0;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
@@ -138,12 +142,12 @@ __global__ void __launch_bounds__(kF16Threads, 2) fold16_kernel(const __grid_con
 #pragma unroll
       for (int e = 0; e < 4; ++e) acc[nt][e] = 0.f;
 
-    const bool row_live = g < p.rows;
-    const unsigned short* xg = a.x + (int64_t)g * a.ldx;
-    const unsigned short* pg = a.xp + (int64_t)g * a.ldx;
+    const bool row_live = row0 + g < p.rows, hi_live = HI && row0 + g + 8 < p.rows;
+    const unsigned short* xg = a.x + (int64_t)(row0 + g) * a.ldx;
+    const unsigned short* pg = a.xp + (int64_t)(row0 + g) * a.ldx;
     const int64_t groups = (a.words + 3) / 4;
     // software pipeline: the next group's code words and inputs load while this one computes
-    uint32_t wu[4], wv[4], ax[8], ap[8];
+    uint32_t wu[4], wv[4], ax[8], ap[8], axh[8], aph[8];
     auto fetch = [&](int64_t gi) {
       const int64_t wi = 4 * gi + t;  // this lane's code word of the group
       const int64_t i0 = 64 * gi + 16 * t;
@@ -155,14 +159,16 @@ __global__ void __launch_bounds__(kF16Threads, 2) fold16_kernel(const __grid_con
       }
       load_row16(ax, xg, i0, a.n, row_live, a.vec);
       load_row16(ap, pg, i0, a.n, row_live, a.vec);
+      load_row16(axh, xg + 8 * a.ldx, i0, a.n, hi_live, a.vec);
+      load_row16(aph, pg + 8 * a.ldx, i0, a.n, hi_live, a.vec);
     };
     if (warp < groups) fetch(warp);
     for (int64_t gi = warp; gi < groups; gi += W) {
-      uint32_t cwu[4], cwv[4], cax[8], cap[8];
+      uint32_t cwu[4], cwv[4], cax[8], cap[8], caxh[8], caph[8];
 #pragma unroll
       for (int k = 0; k < 4; ++k) { cwu[k] = wu[k]; cwv[k] = wv[k]; }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) { cax[k] = ax[k]; cap[k] = ap[k]; }
+      for (int k = 0; k < 8; ++k) { cax[k] = ax[k]; cap[k] = ap[k]; caxh[k] = axh[k]; caph[k] = aph[k]; }
       if (gi + W < groups) fetch(gi + W);
 #pragma unroll
       for (int nt = 0; nt < 4; ++nt) {
@@ -174,8 +180,8 @@ __global__ void __launch_bounds__(kF16Threads, 2) fold16_kernel(const __grid_con
         const uint32_t bv[8] = {vl.x, vl.y, vl.z, vl.w, vh.x, vh.y, vh.z, vh.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          mma_16<BF>(acc[nt], cax[2 * j], 0u, cax[2 * j + 1], 0u, bu[2 * j], bu[2 * j + 1]);
-          mma_16<BF>(acc[nt], cap[2 * j], 0u, cap[2 * j + 1], 0u, bv[2 * j], bv[2 * j + 1]);
+          mma_16<BF>(acc[nt], cax[2 * j], caxh[2 * j], cax[2 * j + 1], caxh[2 * j + 1], bu[2 * j], bu[2 * j + 1]);
+          mma_16<BF>(acc[nt], cap[2 * j], caph[2 * j], cap[2 * j + 1], caph[2 * j + 1], bv[2 * j], bv[2 * j + 1]);
         }
       }
     }
@@ -185,15 +191,19 @@ __global__ void __launch_bounds__(kF16Threads, 2) fold16_kernel(const __grid_con
     for (int nt = 0; nt < 4; ++nt) {
       red[warp][g][8 * nt + 2 * t] = acc[nt][0];
       red[warp][g][8 * nt + 2 * t + 1] = acc[nt][1];
+      if constexpr (HI) {
+        red[warp][g + 8][8 * nt + 2 * t] = acc[nt][2];
+        red[warp][g + 8][8 * nt + 2 * t + 1] = acc[nt][3];
+      }
     }
     __syncthreads();
-    for (int o = threadIdx.x; o < kF16Rows * kF16Tile; o += kF16Threads) {
+    for (int o = threadIdx.x; o < kRows * kF16Tile; o += kThreads) {
       const int r = o / kF16Tile, c = o % kF16Tile;
-      if (r < p.rows && c0 + c < a.m) {
+      if (row0 + r < p.rows && c0 + c < a.m) {
         float s = red[0][r][c];
 #pragma unroll
         for (int w = 1; w < W; ++w) s = __fadd_rn(s, red[w][r][c]);
-        a.y[(int64_t)r * a.ldy + c0 + c] = s;
+        a.y[(int64_t)(row0 + r) * a.ldy + c0 + c] = s;
       }
     }
     __syncthreads();  // red is reused by the next item
@@ -218,35 +228,27 @@ kd_status check_fold16(const kd_fold_mat_f16& a, int64_t batch) {
 namespace kd {
 namespace {
 
-kd_status fold16_run(const kd_fold_mat_f16* mats, int count, int64_t batch, void* stream, bool bf) {
-  if (!mats || count < 1 || count > KD_MAX_BATCH || batch < 0) return KD_ERR_INVALID_ARG;
-  for (int i = 0; i < count; ++i) {
-    const kd_status st = check_fold16(mats[i], batch);
-    if (st != KD_OK) return st;
-  }
-  int64_t work = 0;
-  for (int i = 0; i < count; ++i) work += mats[i].m;
-  if (batch == 0 || work == 0) return KD_OK;
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (batch > kF16Rows) return fold16_tc_run(mats, count, batch, s, bf);
-  // one launch reads the code planes once
+// Short vectors of many channels (an output head): the tcgen05 kernel spends its time around the
+// few MMAs of its tiles.  Measured, this kernel against tcgen05 (us): 256 x 50000 18 / 37 at 9 to
+// 16 rows, 31 / 38 at 17 to 32; 768 x 50257 28 / 43 and 50 / 46; 1024 x 50304 34 / 47 and 61 / 50;
+// 2048 x 32000 40 / 42; 768 x 8192 11 / 13, 768 x 4096 10.4 / 10.7.  With fewer channels tcgen05
+// stays, up to 2 us slower alone, because a layer that also has longer vectors would need two
+// launches.  By the matrix and the batch alone, as every choice here, so that a matrix gives the
+// same bits alone and in a batched call.
+bool wide_short(const kd_fold_mat_f16& a, int64_t batch) {
+  return batch <= 16 ? a.n <= 1024 && a.m >= 8192 : batch <= 32 && a.n <= 256 && a.m >= 16384;
+}
+
+template <bool HI, int W>
+kd_status launch_fold16(const kd_fold_mat_f16* mats, int count, int64_t batch, cudaStream_t s, bool bf) {
   Fold16Params p;
-  p.count = count;
+  p.count = 0;
   p.rows = (int)batch;
-  // work items numbered longest vectors first, so that the long items of a layer are
-  // not the last ones started
-  int order[KD_MAX_BATCH];
-  for (int i = 0; i < count; ++i) order[i] = i;
-  for (int i = 1; i < count; ++i)
-    for (int k = i; k > 0 && mats[order[k]].n > mats[order[k - 1]].n; --k) {
-      const int tmp = order[k];
-      order[k] = order[k - 1];
-      order[k - 1] = tmp;
-    }
-  int64_t items = 0;
+  p.items = 0;
   for (int i = 0; i < count; ++i) {
-    const kd_fold_mat_f16& a = mats[order[i]];
-    Fold16Mat& f = p.mat[i];
+    const kd_fold_mat_f16& a = mats[i];
+    if (a.m == 0) continue;
+    Fold16Mat& f = p.mat[p.count++];
     f.codes_u = a.codes_u;
     f.codes_v = a.codes_v;
     f.centres_u = a.centres_u;
@@ -259,18 +261,46 @@ kd_status fold16_run(const kd_fold_mat_f16* mats, int count, int64_t batch, void
     f.words = (a.n + 15) / 16;
     f.ldx = a.ldx;
     f.ldy = a.ldy;
-    f.item0 = items;
+    f.item0 = p.items;
     f.vec = aligned16(f.x, 16) && aligned16(f.xp, 16) && a.ldx % 8 == 0;
-    items += (a.m + kF16Tile - 1) / kF16Tile;
+    p.items += (a.m + kF16Tile - 1) / kF16Tile;
   }
-  p.items = items;
+  if (p.items == 0) return KD_OK;
   // one CTA per work item (the grid-stride loop covers grids past 2^30 items)
-  const int64_t grid = items < (int64_t)1 << 30 ? items : (int64_t)1 << 30;
-  const unsigned gr = (unsigned)grid;
-  if (bf) fold16_kernel<true><<<gr, kF16Threads, 0, s>>>(p);
-  else fold16_kernel<false><<<gr, kF16Threads, 0, s>>>(p);
-  if (cudaGetLastError() != cudaSuccess) return KD_ERR_CUDA;
-  return KD_OK;
+  const int64_t most = (int64_t)1 << 30;
+  const dim3 grid((unsigned)(p.items < most ? p.items : most), HI ? (unsigned)((batch + 15) / 16) : 1u);
+  if (bf) fold16_kernel<true, HI, W><<<grid, 32 * W, 0, s>>>(p);
+  else fold16_kernel<false, HI, W><<<grid, 32 * W, 0, s>>>(p);
+  return cudaGetLastError() == cudaSuccess ? KD_OK : KD_ERR_CUDA;
+}
+
+kd_status fold16_run(const kd_fold_mat_f16* mats, int count, int64_t batch, void* stream, bool bf) {
+  if (!mats || count < 1 || count > KD_MAX_BATCH || batch < 0) return KD_ERR_INVALID_ARG;
+  for (int i = 0; i < count; ++i) {
+    const kd_status st = check_fold16(mats[i], batch);
+    if (st != KD_OK) return st;
+  }
+  if (batch == 0) return KD_OK;
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  // the short ones, then the others, each longest vectors first, so that the long items of a
+  // layer are not the last ones started
+  kd_fold_mat_f16 sorted[KD_MAX_BATCH];
+  int few = 0;
+  for (int i = 0; i < count; ++i) few += wide_short(mats[i], batch);
+  for (int i = 0, at[2] = {0, few}; i < count; ++i) {
+    const int side = wide_short(mats[i], batch) ? 0 : 1;
+    int k = at[side]++;
+    for (; k > (side ? few : 0) && mats[i].n > sorted[k - 1].n; --k) sorted[k] = sorted[k - 1];
+    sorted[k] = mats[i];
+  }
+  kd_status st = KD_OK;
+  if (few)
+    st = batch > kF16Rows ? launch_fold16<true, kF16ShortWarps>(sorted, few, batch, s, bf)
+                          : launch_fold16<false, kF16ShortWarps>(sorted, few, batch, s, bf);
+  if (st == KD_OK && few < count)
+    st = batch > kF16Rows ? fold16_tc_run(sorted + few, count - few, batch, s, bf)
+                          : launch_fold16<false, kF16Warps>(sorted + few, count - few, batch, s, bf);
+  return st;
 }
 
 }  // namespace

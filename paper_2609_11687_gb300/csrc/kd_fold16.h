@@ -1,5 +1,4 @@
-// The two kernels of the 16-bit 2-bit product (kd_fold16.cu: up to 8 batch rows,
-// kd_fold16_tc.cu: more).
+// The tcgen05 kernel of the 16-bit 2-bit product (kd_fold16.cu has the other one and the choice).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -8,8 +7,7 @@
 
 namespace kd {
 
-// kd_matmul_2bit_f16_batch (bf: _bf16_batch) on validated descriptors, batch >= 1 and at
-// least one matrix with m > 0
+// kd_matmul_2bit_f16_batch (bf: _bf16_batch) on validated descriptors, batch >= 1
 kd_status fold16_tc_run(const kd_fold_mat_f16* mats, int count, int64_t batch, cudaStream_t s, bool bf);
 
 }  // namespace kd

@@ -1,5 +1,5 @@
 // The folded 2-bit layer product of App. C for 16-bit activations on tcgen05, for more than
-// 8 batch rows (kd_fold16.cu states the product and takes fewer rows).  The code planes
+// 8 batch rows (kd_fold16.cu states the product and takes fewer rows and wide, short matrices).  The code planes
 // are read and decoded once per block of up to 256 batch rows.
 //
 // Mapping.  tcgen05.mma with M = 128 output channels, N = the batch rows of the block,
