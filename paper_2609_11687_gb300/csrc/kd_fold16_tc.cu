@@ -38,6 +38,7 @@
 #include "kd_dec16.cuh"
 #include "kd_fold16.h"
 #include "kd_tc.cuh"
+#include "kd_tc_host.h"
 
 namespace kd {
 namespace {
@@ -204,6 +205,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
     if (TMA) {
       int s = 0;
       uint32_t par = 1;  // the first round finds every slot free
+      int issued = 0;
       for (int i = 0; i < L * (2 / BH); ++i) {
         if (i >= S && !ctl_wait(&ctl, &ctl.empty_b[s], par)) break;
         if (elect_one()) {
@@ -216,10 +218,17 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
           for (int h = 0; h < BH; ++h) tma_load_2d(dst + h * bstage, map, x + h * kStageK, row0, &ctl.full_b[s]);
         }
         __syncwarp();
+        ++issued;
         if (++s == S) {
           s = 0;
           par ^= 1;
         }
+      }
+      // shared memory is not used otherwise, nor given back, before the copies have landed, also
+      // after an expired wait (bounded as well)
+      for (s = 0; s < S; ++s) {
+        const int last = ring_last_parity(issued, S, s);
+        if (last >= 0 && !mbar_wait_bounded(&ctl.full_b[s], last)) *(volatile int*)&ctl.fail = 1;
       }
     }
   } else if (warp == kDecWarps + 1) {
@@ -342,17 +351,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
     while (done < chunks) promote();
   }
 
-  // Every MMA has completed and every copy has landed (the accumulators were waited for).
-  // After an expired wait: let the copies in flight land, bounded, before shared memory goes.
-  if (*(volatile int*)&ctl.fail && threadIdx.x == 0 && TMA) {
-    for (int s = 0; s < S; ++s) {
-      const long long t0 = clock64();
-      while (!mbar_try_wait(&ctl.full_b[s], 0) && !mbar_try_wait(&ctl.full_b[s], 1) && clock64() - t0 < kWaitCycles) {
-      }
-    }
-  }
   __syncthreads();
-  const float bad = *(volatile int*)&ctl.fail ? __int_as_float(0x7FC00000) : 0.f;
   const int cols = p.rows - row0 < nt ? p.rows - row0 : nt;  // batch rows of this block
   if (p.split == 1) {
     if (warp < kDecWarps) {
@@ -361,7 +360,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
 #pragma unroll
         for (int i = 0; i < NC; ++i) {
           const int c = (warp >> 2) * NC + i;
-          if (c < cols) a.y[(int64_t)(row0 + c) * a.ldy + j] = __fadd_rn(acc[i], bad);
+          if (c < cols) a.y[(int64_t)(row0 + c) * a.ldy + j] = acc[i];
         }
       }
     }
@@ -372,9 +371,7 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
 #pragma unroll
       for (int i = 0; i < NC; ++i) {
         const int c = (warp >> 2) * NC + i;
-        if (c < cols)
-          asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + ch) * 4), "f"(__fadd_rn(acc[i], bad))
-                       : "memory");
+        if (c < cols) asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + ch) * 4), "f"(acc[i]) : "memory");
       }
     }
     cluster_sync_all();
@@ -386,6 +383,11 @@ __global__ void __launch_bounds__(kThreads, tc_ctas(NTC)) fold16_tc_kernel(const
       }
     }
     cluster_sync_all();  // the peers' reads of this CTA's shared memory are done
+  }
+  if (*(volatile int*)&ctl.fail) {  // over whatever the tile's CTAs have written
+    __syncthreads();
+    for (int c = warp >> 2; live && c < cols; c += 4)
+      a.y[(int64_t)(row0 + c) * a.ldy + c0 + r] = __int_as_float(0x7FC00000);
   }
   if (warp == kDecWarps + 1) tmem_dealloc(tmem, kCols);
 }
