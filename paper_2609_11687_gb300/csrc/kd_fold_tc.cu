@@ -98,7 +98,7 @@ struct FoldTcParams {
 };
 
 struct Ctl {
-  uint64_t full_a[kSlotsA], empty_a[kSlotsA], full_b[kSlotsB], empty_b[kSlotsB], acc_full, acc_empty;
+  uint64_t full_a[kSlotsA], empty_a[kSlotsA], full_b[kSlotsB], empty_b[kSlotsB], acc_full, acc_empty, drained;
   uint32_t tmem;
   int fail;   // a wait expired: the tile's outputs become NaN
   uint32_t row_max[kRows];  // bits of the largest finite magnitude
@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
     }
     if (lane == 0) {
       mbar_init(&ctl.acc_full, 1);
+      mbar_init(&ctl.drained, 1);
       mbar_init(&ctl.acc_empty, kDecWarps);
       ctl.fail = 0;
       ctl.nan_rows = ctl.inf_rows = ctl.infs = 0u;
@@ -345,18 +346,17 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
   for (int k = 0; k < 8; ++k) acc[k] = 0.f;
   if (warp == kDecWarps + kSplitWarps) {
     // ---- MMAs ----
-    const uint32_t idesc = tc_idesc(true, nt);
-    const uint64_t db0 = tc_desc(ring);
-    int in_pass = 0, in_chunk = 0, chunk = 0;
-    bool ok = true;
-    for (int i = 0; i < V && ok; ++i) {
-      if (in_chunk == 0 && chunk > 0) ok = ctl_wait(ctl, &ctl.acc_empty, (chunk - 1) & 1);
-      const int sa = i % kSlotsA, sb = i % kSlotsB;
-      ok = ok && ctl_wait(ctl, &ctl.full_b[sb], (i / kSlotsB) & 1);
-      ok = ok && ctl_wait(ctl, &ctl.full_a[sa], (i / kSlotsA) & 1);
-      tc_fence_after();
-      const bool end = in_chunk == kChunk - 1 || in_pass == L - 1;
-      if (ok && elect_one()) {
+    if (elect_one()) {
+      const uint32_t idesc = tc_idesc(true, nt);
+      const uint64_t db0 = tc_desc(ring);
+      int in_pass = 0, in_chunk = 0, chunk = 0;
+      for (int i = 0; i < V; ++i) {
+        const int sa = i % kSlotsA, sb = i % kSlotsB;
+        if ((in_chunk == 0 && chunk > 0 && !ctl_wait(ctl, &ctl.acc_empty, (chunk - 1) & 1)) ||
+            !ctl_wait(ctl, &ctl.full_b[sb], (i / kSlotsB) & 1) || !ctl_wait(ctl, &ctl.full_a[sa], (i / kSlotsA) & 1))
+          break;
+        tc_fence_after();
+        const bool end = in_chunk == kChunk - 1 || in_pass == L - 1;
         const uint32_t ta = tmem + 128 + 64 * sa;
         const uint64_t db = db0 + (uint64_t)(sb * (kBBytes >> 4));
 #pragma unroll
@@ -367,16 +367,17 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
         tc_commit(&ctl.empty_a[sa]);
         tc_commit(&ctl.empty_b[sb]);
         if (end) tc_commit(&ctl.acc_full);
+        ++in_chunk;
+        ++in_pass;
+        if (end) {
+          in_chunk = 0;
+          ++chunk;
+          if (in_pass == L) in_pass = 0;
+        }
       }
-      __syncwarp();
-      ++in_chunk;
-      ++in_pass;
-      if (end) {
-        in_chunk = 0;
-        ++chunk;
-        if (in_pass == L) in_pass = 0;
-      }
+      tc_drain(&ctl.drained, &ctl.fail);
     }
+    __syncwarp();
   } else if (warp >= kDecWarps) {
     // ---- B tiles: thread (row t / 8 + 8 h, inputs 8 (t % 8) .. + 7), h = 0, 1 ----
     const int sg = (warp - kDecWarps) >> 1;
@@ -546,7 +547,7 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
     while (done < chunks * reps) promote();
   }
 
-  __syncthreads();  // the MMAs have completed (their sums were waited for): shared memory is free
+  __syncthreads();  // the MMAs have completed: shared memory is free
   const float bad = *(volatile int*)&ctl.fail ? __int_as_float(0x7FC00000) : 0.f;
   if (warp < kDecWarps) {
     auto centre = [&](int i) {  // of input i

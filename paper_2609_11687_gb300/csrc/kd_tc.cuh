@@ -71,6 +71,14 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                : "memory");
 }
 
+// Waits, bounded, until every tcgen05.mma that this thread issued has completed; `bar` (one
+// arrival) serves this alone.  Before shared memory or TMEM is used for anything else or given
+// back: after an expired wait nobody has waited for the sums.
+__device__ __forceinline__ void tc_drain(uint64_t* bar, int* fail) {
+  tc_commit(bar);
+  if (!mbar_wait_bounded(bar, 0)) *(volatile int*)fail = 1;
+}
+
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -112,8 +120,13 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 // this CTA has taken kWaitTries tries (every later one then gives up at once).  A try parks the
 // thread for some hundred cycles at most, so the limit is near a second.  The loop is a try, a
 // counter and two branches: with a clock and a flag read in it, polling took a fifth of the
-// instructions of the whole kernel.
-constexpr uint32_t kWaitTries = 1u << 22;
+// instructions of the whole kernel.  Lanes of a warp may get different answers, and lanes that
+// gave up would leave the others in a later elect.sync, without limit: a warp that elects a lane
+// after its waits votes on them first.
+#ifndef KD_WAIT_TRIES
+#define KD_WAIT_TRIES (1u << 22)
+#endif
+constexpr uint32_t kWaitTries = KD_WAIT_TRIES;
 __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* fail) {
   if (mbar_try_wait(bar, parity)) return true;
   if (*(volatile int*)fail) return false;
