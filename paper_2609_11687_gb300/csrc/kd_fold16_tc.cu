@@ -437,7 +437,8 @@ cudaError_t launch_tc(FoldTcParams& p, int64_t tiles, cudaStream_t s) {
   const int left = budget / slot;
   p.slots_b = left < kMaxB ? left : kMaxB;
   // at least what the partial tiles of a split take at the end
-  const size_t smem = (size_t)p.slots_b * slot + 1024;
+  const int used = p.slots_b * slot + 1024, least = tc_smem_floor(tc_cols(NTC));
+  const size_t smem = (size_t)(used > least ? used : least);
   auto kernel = fold16_tc_kernel<BF, NTC, TMA>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

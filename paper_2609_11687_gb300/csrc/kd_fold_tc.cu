@@ -54,6 +54,7 @@
 #include "kd_dec16.cuh"
 #include "kd_fold_tc.h"
 #include "kd_tc.cuh"
+#include "kd_tc_host.h"
 
 namespace kd {
 namespace {
@@ -68,8 +69,9 @@ constexpr int kSplitWarps = 4;  // two groups of two
 constexpr int kThreads = 32 * (kDecWarps + kSplitWarps + 1);
 constexpr int kSlotsA = 2, kSlotsB = 4;    // A in TMEM, B in shared memory
 constexpr int kBBytes = kDigits * kRows * 128;
-constexpr int kSmem = kSlotsB * kBBytes + 1024;
 constexpr uint32_t kCols = 256;            // TMEM: sums of plane p at 64 p, A slot s at 128 + 64 s (32 per plane)
+constexpr int kSmem = tc_smem_floor(kCols);
+static_assert(kSlotsB * kBBytes + 1024 <= kSmem, "the B slots fit");
 constexpr uint32_t kBig = 0x72000000u;     // bits of 2^101
 constexpr uint32_t kInf = 0x7F800000u;
 constexpr int kTopExp = 100;               // the sums take at most 2^100 of the row's 2^k before the centres

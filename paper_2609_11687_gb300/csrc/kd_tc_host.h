@@ -18,4 +18,13 @@ KD_TC_HD constexpr int ring_last_parity(int issued, int slots, int s) {
   return s < issued ? ((issued - 1 - s) / slots) & 1 : -1;
 }
 
+// Dynamic shared memory that a CTA with `cols` columns of TMEM (256 or 512 of the SM's 512) asks
+// for at least.  CTAs whose shared memory fits on an SM together then have their columns there
+// too, whichever of the kernels and streams they come from: three of 256, or 256 beside 512, do
+// not fit (228 KB per SM, 1 KB of it reserved per CTA).  Otherwise tcgen05.alloc would wait for a
+// resident CTA to end, and two clusters that hold columns on one SM and want them on another
+// would wait for each other at their cluster barriers.
+constexpr int kSmemPerSM = 228 * 1024;
+KD_TC_HD constexpr int tc_smem_floor(int cols) { return kSmemPerSM / 768 * cols; }
+
 }  // namespace kd

@@ -13,6 +13,8 @@ CSRC = os.path.join(os.path.dirname(__file__), "..", "paper_2609_11687_gb300", "
 SHIM = r"""
 #include "kd_tc_host.h"
 extern "C" int last_parity(int issued, int slots, int s) { return kd::ring_last_parity(issued, slots, s); }
+extern "C" int smem_floor(int cols) { return kd::tc_smem_floor(cols); }
+extern "C" int smem_per_sm() { return kd::kSmemPerSM; }
 """
 
 
@@ -59,3 +61,18 @@ def test_ring_drain_waits_for_every_copy(lib):
                     assert bars[s].reads_complete(parity) == (s not in missing)
                     # either parity, as a loop's end, would not have waited
                     assert bars[s].reads_complete(0) or bars[s].reads_complete(1)
+
+
+def test_ctas_that_fit_on_an_sm_have_their_tmem_there(lib):
+    """Any set of CTAs of 256 and 512 columns whose shared memory fits (1 KB reserved each, at
+    least the floor of dynamic memory) needs no more than the SM's 512 columns; two of 256 or one
+    of 512 do fit, beside 2 KB of static memory."""
+    total = lib.smem_per_sm()
+    assert total == 228 * 1024
+    size = {c: lib.smem_floor(c) + 1024 for c in (256, 512)}
+    for a in range(8):
+        for b in range(4):
+            if a * size[256] + b * size[512] <= total:
+                assert 256 * a + 512 * b <= 512, (a, b)
+    assert 2 * (size[256] + 2048) <= total and size[512] + 2048 <= total
+    assert all(lib.smem_floor(c) <= 227 * 1024 for c in (256, 512))
