@@ -315,11 +315,17 @@ def _torch():
 _PACKERS = {}
 
 
-def _pack(fields: str, count: int, values) -> bytes:
-    key = (fields, count)
+_CODES = {ctypes.c_void_p: "Q", ctypes.c_uint64: "Q", ctypes.c_int64: "q"}
+
+
+def _pack(cls, count: int, values) -> bytes:
+    """`count` descriptors of the ctypes structure `cls`, their fields' values in order."""
+    key = (cls, count)
     st = _PACKERS.get(key)
     if st is None:
-        st = _PACKERS[key] = struct.Struct(fields * count)
+        st = struct.Struct("".join(_CODES[t] for _, t in cls._fields_) * count)
+        assert st.size == ctypes.sizeof(cls) * count
+        _PACKERS[key] = st
     return st.pack(*values)
 
 
@@ -462,7 +468,7 @@ def decompose_batch(ws, iters: int, sign_seeds, layout: str = "rows", coeffs: bo
                  o.centres_u.data_ptr(), o.centres_v.data_ptr(), _ptr(o.coeffs) or 0)
         res.append(o)
     wsp = workspace if workspace is not None else Workspace(n, ws[0].device, count=len(ws))
-    st = kd_decompose_batch(_pack("QqqQQQQQQ", len(ws), vals), len(ws), _dtype_code(dt), lay, n, int(iters),
+    st = kd_decompose_batch(_pack(KdMatrix, len(ws), vals), len(ws), _dtype_code(dt), lay, n, int(iters),
                             int(kmeans_iters), wsp.ptr, wsp.nbytes, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_decompose_batch")
@@ -515,9 +521,6 @@ def kd_matmul_2bit_bf16_batch(mats, count, batch, stream) -> int:
     return lib.kd_matmul_2bit_bf16_batch(mats, count, batch, stream)
 
 
-_FOLD_FIELDS = "QQQQQQQqqqq"  # kd_fold_mat, kd_fold_mat_f16
-
-
 def _fold_fields(decs, xs, xps, outs, b, dt, message):
     """The fields of a product's descriptors and its outputs, the inputs checked."""
     torch = _torch()
@@ -560,7 +563,7 @@ def matmul_2bit_f16_batch(decs, xs, xps, outs=None, stream=None):
     vals, res = _fold_fields(decs, xs, xps, outs, b, dt,
                              "x and xp must be 16-bit (batch, n) tensors of one type and shape, unit inner stride")
     call = kd_matmul_2bit_bf16_batch if dt == torch.bfloat16 else kd_matmul_2bit_f16_batch
-    st = call(_pack(_FOLD_FIELDS, len(decs), vals), len(decs), b, _stream(stream))
+    st = call(_pack(KdFoldMatF16, len(decs), vals), len(decs), b, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_matmul_2bit_bf16_batch" if dt == torch.bfloat16 else "kd_matmul_2bit_f16_batch")
     return res
@@ -579,7 +582,7 @@ def matmul_2bit_batch(decs, xs, xps, outs=None, stream=None):
     b = xs[0].shape[0]
     vals, res = _fold_fields(decs, xs, xps, outs, b, torch.float32,
                              "x and xp must be fp32 (batch, n) tensors of one shape, unit inner stride")
-    st = kd_matmul_2bit_batch(_pack(_FOLD_FIELDS, len(decs), vals), len(decs), b, _stream(stream))
+    st = kd_matmul_2bit_batch(_pack(KdFoldMat, len(decs), vals), len(decs), b, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_matmul_2bit_batch")
     return res
@@ -608,7 +611,7 @@ def apply_p_batch(xs, sign_seeds, outs=None, workspace: Optional[Workspace] = No
     n = xs[0].shape[1]
     vals, res = _pmat_fields(xs, outs, n, sign_seeds)
     ws = workspace if workspace is not None else Workspace(n, xs[0].device, count=len(xs))
-    st = kd_apply_p_batch(_pack("QQqQ", len(xs), vals), len(xs), n, ws.ptr, ws.nbytes, _stream(stream))
+    st = kd_apply_p_batch(_pack(KdPMat, len(xs), vals), len(xs), n, ws.ptr, ws.nbytes, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_apply_p_batch")
     return res
@@ -643,7 +646,7 @@ def apply_p_prepared(xs, workspace: Workspace, outs=None, stream=None):
         raise ValueError(f"1..{KD_MAX_BATCH} matrices")
     n = xs[0].shape[1]
     vals, res = _pmat_fields(xs, outs, n, None)
-    st = kd_apply_p_prepared(_pack("QQqQ", len(xs), vals), len(xs), n, workspace.ptr, workspace.nbytes,
+    st = kd_apply_p_prepared(_pack(KdPMat, len(xs), vals), len(xs), n, workspace.ptr, workspace.nbytes,
                              _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_apply_p_prepared")
@@ -761,7 +764,7 @@ def dequantise_batch(planes, n: int, dtype=None, layout: str = "rows", outs=None
             raise ValueError("outputs must share one dtype")
         vals += (codes.data_ptr(), centres.data_ptr(), o.data_ptr(), m, _ld(o))
         res.append(o)
-    st = kd_dequantise_batch(_pack("QQQqq", len(planes), vals), len(planes), n, _dtype_code(dtype), lay,
+    st = kd_dequantise_batch(_pack(KdPlane, len(planes), vals), len(planes), n, _dtype_code(dtype), lay,
                              _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_dequantise_batch")
@@ -828,7 +831,7 @@ def reconstruct_batch(decs, n: int, sign_seeds, dtype=None, layout: str = "rows"
                  int(sign_seeds[i]) & _M64, o.data_ptr(), m, _ld(o))
         res.append(o)
     ws = workspace if workspace is not None else Workspace(n, dev, count=len(decs))
-    st = kd_reconstruct_batch(_pack("QQQQQQqq", len(decs), vals), len(decs), n, _dtype_code(dtype), lay, ws.ptr,
+    st = kd_reconstruct_batch(_pack(KdRecMat, len(decs), vals), len(decs), n, _dtype_code(dtype), lay, ws.ptr,
                               ws.nbytes, _stream(stream))
     if st != KD_OK:
         raise KashinError(st, "kd_reconstruct_batch")
