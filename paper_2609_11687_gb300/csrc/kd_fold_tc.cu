@@ -572,23 +572,40 @@ __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_const
       for (int k = 0; k < 8; ++k)
         if (row == 8 * grp + k) acc[k] = __fadd_rn(acc[k], add);
     }
-    const uint32_t plain = of & (plain_channel ? ~0u : many ? ctl.inf_rows : 0u);
-    if (live && plain) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k)
-        if ((plain >> (8 * grp + k)) & 1u) acc[k] = 0.f;
-      for (int i = 0; i < n; ++i) {
-        const float c = centre(i);
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-          if ((plain >> (8 * grp + k)) & 1u) acc[k] = __fmaf_rn(c, __ldg(q + (int64_t)(8 * grp + k) * a.ldx + i), acc[k]);
-      }
-    }
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int c = 8 * grp + k;
       const float nan = (ctl.nan_rows >> c) & 1u ? __int_as_float(0x7FC00000) : bad;
       asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + r) * 4), "f"(__fadd_rn(acc[k], nan)) : "memory");
+    }
+    // plain sums of this channel, a code word and its 16 inputs at a time
+    const uint32_t plain = !live ? 0u : of & (plain_channel ? ~0u : many ? ctl.inf_rows : 0u);
+    for (uint32_t left = plain; left; left &= left - 1) {
+      const int c = __ffs(left) - 1;
+      const float* x = q + (int64_t)c * a.ldx;
+      float sum[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int w = 0; w < words; ++w) {
+        const uint32_t code = __ldg(code_row + w);
+        float f[16];
+#pragma unroll
+        for (int e = 0; e < 16; e += 4) {
+          const int i = 16 * w + e;
+          if (a.vec_x && i < n) {
+            const float4 v = __ldg(reinterpret_cast<const float4*>(x + i));
+            f[e] = v.x; f[e + 1] = v.y; f[e + 2] = v.z; f[e + 3] = v.w;
+          } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) f[e + k] = i + k < n ? __ldg(x + i + k) : 0.f;
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const float lo = (code >> (2 * e)) & 1u ? cen.y : cen.x, hi = (code >> (2 * e)) & 1u ? cen.w : cen.z;
+          if (16 * w + e < n) sum[e & 3] = __fmaf_rn((code >> (2 * e)) & 2u ? hi : lo, f[e], sum[e & 3]);
+        }
+      }
+      const float all = __fadd_rn(__fadd_rn(sum[0], sum[1]), __fadd_rn(sum[2], sum[3]));
+      asm volatile("st.shared.f32 [%0], %1;" ::"r"(ring + (c * kTile + r) * 4), "f"(__fadd_rn(all, bad)) : "memory");
     }
   }
   cluster_sync_all();

@@ -89,3 +89,23 @@ def test_vectors_beyond_one_accumulation(kd):  # noqa: F811
     xp = torch.rand((batch, n), generator=g, device="cuda") + 1.0
     ref = torch.cat([_y64(dec, x[r:r + 1], xp[r:r + 1]) for r in range(batch)])
     _check(kd.matmul_2bit(dec, x, xp), ref)
+
+
+@pytest.mark.parametrize("n", [300, 1000, 2112])
+@pytest.mark.parametrize("batch", [5, 20])
+def test_channel_with_an_unused_infinite_centre(kd, n, batch):  # noqa: F811
+    """Summed plainly: the code that pads the last word has that centre and stays out; rows at an
+    odd offset give the same."""
+    from tests.test_gpu_fold_tc_centres import _recode
+    dec, x, xp = _case(kd, n, 140, batch)
+    _recode(dec.codes_u, 5, 0, 1)
+    dec.centres_u[5, 0] = -float("inf")
+    y = kd.matmul_2bit(dec, x, xp)
+    ref = dec.centres_u.clone()
+    ref[5, 0] = 0.0
+    y64 = x.double() @ _plane(dec.codes_u, ref, n).t() + xp.double() @ _plane(dec.codes_v, dec.centres_v, n).t()
+    assert torch.isfinite(y).all()
+    assert ((y.double() - y64).abs().amax(1) <= 1e-5 * y64.abs().amax(1)).all()
+    big = torch.zeros((2, batch, n + 9), device="cuda")
+    big[0][:, 1:1 + n], big[1][:, 1:1 + n] = x, xp
+    assert torch.equal(kd.matmul_2bit(dec, big[0][:, 1:1 + n], big[1][:, 1:1 + n]), y)
