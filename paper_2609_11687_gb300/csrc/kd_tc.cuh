@@ -134,7 +134,7 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* fai
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
       "TRY_%=:\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      KD_MBAR_WAIT ".parity.shared::cta.b64 p, [%1], %2;\n\t"
       "@p bra DONE_%=;\n\t"
       "add.u32 %0, %0, -1;\n\t"
       "setp.ne.u32 q, %0, 0;\n\t"

@@ -1,5 +1,5 @@
 """The tensor-core products when waits inside the kernel run out: built here with a limit of one
-try per wait (csrc/kd_tc.cuh), where almost any wait expires.  A call returns, each output is
+try per wait that does not park the thread (csrc/kd_tc.cuh), where almost any wait expires.  A call returns, each output is
 NaN or right to the bit, and the device works on as before."""
 
 import ctypes
@@ -20,7 +20,8 @@ def impatient(tmp_path_factory):
     from paper_2609_11687_gb300 import build
     so = str(tmp_path_factory.mktemp("impatient") / "lib.so")
     srcs = [os.path.join(build.CSRC, f) for f in ("kd_fold.cu", "kd_fold_tc.cu", "kd_fold16.cu", "kd_fold16_tc.cu")]
-    subprocess.run([build._nvcc()] + build.NVCC_FLAGS + ["-DKD_WAIT_TRIES=1", "-shared", "-o", so] + srcs, check=True)
+    subprocess.run([build._nvcc()] + build.NVCC_FLAGS + ["-DKD_WAIT_TRIES=1", '-DKD_MBAR_WAIT="mbarrier.test_wait"',
+                    "-shared", "-o", so] + srcs, check=True)
     return ctypes.CDLL(so)
 
 
