@@ -26,6 +26,7 @@
 
 #include "kashin.h"
 #include "kd_fold_tc.h"
+#include "kd_tc.cuh"
 
 namespace kd {
 namespace {
@@ -183,10 +184,13 @@ __global__ void __launch_bounds__(kFoldThreads, 2) fold_kernel(const __grid_cons
       if (j0 + r < a.m && row0 + b < p.rows) a.y[(int64_t)(row0 + b) * a.ldy + j0 + r] = t;
     }
   }
+  grid_dependency_wait();  // no dependency: nothing to wait for
 }
 
+// beside: the launch ahead on the stream is the tensor-core kernel of the call's other matrices;
+// this one needs nothing of it and runs beside it, and ends after it (the kernel's last wait).
 template <int B, bool MANY>
-cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
+cudaError_t launch_fold(const FoldParams& p, bool beside, cudaStream_t s) {
   int dev = 0, sms = 0, per = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -195,8 +199,16 @@ cudaError_t launch_fold(const FoldParams& p, cudaStream_t s) {
     return e;
   if (per < 1) return cudaErrorInvalidConfiguration;
   const int64_t grid = p.items < (int64_t)per * sms ? p.items : (int64_t)per * sms;
-  fold_kernel<B, MANY><<<dim3((unsigned)grid, (unsigned)((p.rows + B - 1) / B)), kFoldThreads, 0, s>>>(p);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, (unsigned)((p.rows + B - 1) / B));
+  cfg.blockDim = dim3(kFoldThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = beside ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fold_kernel<B, MANY>, p);
 }
 
 bool aligned(const void* ptr, size_t a) { return reinterpret_cast<uintptr_t>(ptr) % a == 0; }
@@ -224,7 +236,7 @@ namespace kd {
 namespace {
 
 template <int B>
-kd_status fold_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStream_t s) {
+kd_status fold_run(const kd_fold_mat* mats, int count, int64_t batch, bool beside, cudaStream_t s) {
   constexpr int RT = FoldTile<B>::RT;
   FoldParams p;
   p.count = 0;
@@ -251,7 +263,7 @@ kd_status fold_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStream
     p.items += (a.m + RT - 1) / RT;
   }
   if (p.items == 0) return KD_OK;
-  const cudaError_t e = batch > B ? launch_fold<B, (B > 1)>(p, s) : launch_fold<B, false>(p, s);
+  const cudaError_t e = batch > B ? launch_fold<B, (B > 1)>(p, beside, s) : launch_fold<B, false>(p, beside, s);
   return e == cudaSuccess ? KD_OK : KD_ERR_CUDA;
 }
 
@@ -265,20 +277,22 @@ namespace {
 // a short chain per item; the tensor-core kernel has the same time up to 16 rows and up to about
 // 9000 channels, 11 us at n = 256, 13 at 768, 17 at 2048, 23 at 4096, 44 at 11008 (nearly twice
 // that with centres that are not symmetric).  Measured, lookup against tensor cores (us):
-//   one row     always (7B layer 86)
-//   two rows    4096 x 300 11 / 23, 4096 x 4096 19 / 23, 4096 x 11008 35 / 43, 7B layer 125 / 123
+//   one row     always (7B layer 88)
+//   two rows    4096 x 300 11 / 23, 4096 x 4096 19 / 23, 4096 x 11008 35 / 43, 7B layer 125 / 119
 //               (125 / 217 not symmetric), 768 x 768 10 / 13; short vectors of many channels the
 //               other way: 768 x 4096 15 / 13, 256 x 11008 26 / 17
-//   3, 4 rows   4096 x 300 9 / 23, 4096 x 2048 18 / 23, 4096 x 3072 24 / 23, 11008 x 2048 36 / 44
-//   8, 16 rows  4096 x 1024 18 / 23, 27 / 23; 16384 x 300 18 / 59, 26 / 64
-// Below n = 4096 three rows and more stay with the tensor cores although single matrices would
-// gain up to 8 us (3072 x 768 13 / 19): the layers of such models are called whole, and two
-// launches cost them more (768-wide layer, 4 rows: 21 us in one).  By the matrix and the batch
-// alone, so that a matrix gives the same bits alone and in a batched call.
+//   3, 4 rows   4096 x 300 9 / 23, 4096 x 1024 13 / 23, 4096 x 2048 18 / 23, 11008 x 1024 21 / 44
+//   8, 16 rows  4096 x 300 11 / 23, 12 / 24; 4096 x 1024 18 / 23, 27 / 23; 16384 x 300 18 / 59
+// Alone, three rows and more would gain up to 4096 channel pairs of rows and from n = 1024 on
+// (3072 x 768 at 4 rows 13 / 19), but mostly a layer is one call, where the tensor cores take such
+// a matrix beside the others for less: 4096 x 1024 twice and 4096 x 4096 twice at 8 rows 55 us
+// with the small ones looked up, 42 without; a layer with the former at 4 rows 138 and 128.  So
+// only up to 1024, and from n = 4096 on.  By the matrix and the batch alone, so that a matrix gives the same bits alone and
+// in a batched call.
 bool by_lookup(const kd_fold_mat& a, int64_t batch) {
   if (batch == 1) return true;
   if (batch == 2) return a.n >= 1024 || a.m <= 3072;
-  return batch <= 16 && a.n >= 4096 && a.m <= 4096 && a.m * ((batch + 1) / 2) <= 4096;
+  return batch <= 16 && a.n >= 4096 && a.m <= 1024 && a.m * ((batch + 1) / 2) <= 1024;
 }
 
 }  // namespace
@@ -294,13 +308,17 @@ extern "C" kd_status kd_matmul_2bit_batch(const kd_fold_mat* mats, int count, in
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   kd_fold_mat sorted[KD_MAX_BATCH];
   int few = 0, rest = 0;
+  bool tc = false;  // the tensor-core kernel is launched
   for (int i = 0; i < count; ++i)
     if (kd::by_lookup(mats[i], batch)) sorted[few++] = mats[i];
   for (int i = 0; i < count; ++i)
-    if (!kd::by_lookup(mats[i], batch)) sorted[few + rest++] = mats[i];
-  kd_status st = KD_OK;
-  if (few) st = batch == 1 ? kd::fold_run<1>(sorted, few, batch, s) : kd::fold_run<2>(sorted, few, batch, s);
-  if (st == KD_OK && rest) st = kd::fold_tc_run(sorted + few, rest, batch, s);
+    if (!kd::by_lookup(mats[i], batch)) {
+      sorted[few + rest++] = mats[i];
+      tc = tc || mats[i].m > 0;
+    }
+  kd_status st = tc ? kd::fold_tc_run(sorted + few, rest, batch, s) : KD_OK;
+  if (st == KD_OK && few)
+    st = batch == 1 ? kd::fold_run<1>(sorted, few, batch, tc, s) : kd::fold_run<2>(sorted, few, batch, tc, s);
   return st;
 }
 

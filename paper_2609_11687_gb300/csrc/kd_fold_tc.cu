@@ -190,6 +190,7 @@ __global__ void __launch_bounds__(kGridThreads) row_grid_kernel(const __grid_con
 __global__ void __launch_bounds__(kThreads, 2) fold_tc_kernel(const __grid_constant__ FoldTcParams p) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ Ctl ctl;
+  grid_dependents_start();  // the lookup kernel of the call's other matrices may run beside this one
   const uint32_t ring = (smem_u32(smem_raw) + 1023u) & ~1023u;  // the B slots
   const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
   const int lane = threadIdx.x & 31;

@@ -25,8 +25,10 @@
 // operator M to the frequency pairs in registers and runs their inverse transforms: no pass
 // of its own for M and one exchange less in each direction.
 //
-// Bound by latency (issue 38 %, the first stall is table loads that miss L1) and by the
-// instructions around the arithmetic.  Measured at 16 blocks, before (run-time padding, a pass
+// Bound by latency (issue 38 %, the first stall is table loads that miss L1), by the
+// instructions around the arithmetic, and from n = 1025 to 8192 by spills: two CTAs per SM leave
+// 128 registers a thread, of which E = 10, 20 and 32 spill 96, 840 and 996 bytes (E = 4 and 44
+// none).  Measured at 16 blocks, before (run-time padding, a pass
 // for M, the greedy steps in shared memory, 288 instructions per element and P, half the
 // shared-memory wavefronts conflicts) and now:
 //   n = 640 x 8000 2.75 -> 1.91 ms, 2560 x 6000 4.92 -> 3.29, 5120 x 5120 (columns, 3

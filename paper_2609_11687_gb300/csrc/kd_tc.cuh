@@ -1,7 +1,7 @@
 // Fifth-generation tensor-core building blocks (sm_103a): TMEM allocation, tcgen05.mma
-// on shared-memory operands, its commit, TMEM loads, tiled TMA loads, clusters.
+// (A in TMEM, B in shared memory), its commit, TMEM loads and stores, tiled TMA loads, clusters.
 //
-// Operand tiles are K-major with the 128-byte swizzle: a tile row (one M or N index)
+// B tiles are K-major with the 128-byte swizzle: a tile row (one N index)
 // is 64 16-bit K entries = 128 bytes, 16-byte chunk c of row r sits at
 // 128 r + 16 (c ^ (r & 7)), and tiles start on 1024-byte boundaries.  One
 // tcgen05.mma covers 16 of the 64 K entries (32 bytes along the row).

@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 
 # n, m, batch, whether the lookup kernel takes it
 LINES = [(1024, 3073, 2, True), (1000, 3072, 2, True), (1000, 3073, 2, False),
-         (4096, 2048, 3, True), (4096, 2049, 4, False), (4095, 60, 3, False),
-         (4096, 1365, 5, True), (4096, 513, 16, False), (4096, 512, 15, True), (4096, 16, 17, False),
+         (4096, 512, 3, True), (4096, 513, 4, False), (4095, 60, 3, False),
+         (4096, 341, 5, True), (4096, 129, 16, False), (4096, 128, 15, True), (4096, 16, 17, False),
          (11008, 1, 16, True)]
 
 
