@@ -123,12 +123,23 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
 // instructions of the whole kernel.  Lanes of a warp may get different answers, and lanes that
 // gave up would leave the others in a later elect.sync, without limit: a warp that elects a lane
 // after its waits votes on them first.
+#ifndef KD_MBAR_WAIT  // a build of the tests: test_wait, which does not park the thread
+#define KD_MBAR_WAIT "mbarrier.try_wait"
+#endif
 #ifndef KD_WAIT_TRIES
 #define KD_WAIT_TRIES (1u << 22)
 #endif
 constexpr uint32_t kWaitTries = KD_WAIT_TRIES;
 __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, int* fail) {
-  if (mbar_try_wait(bar, parity)) return true;
+  uint32_t done;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t" KD_MBAR_WAIT
+      ".parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(done)
+      : "r"(smem_u32(bar)), "r"(parity)
+      : "memory");
+  if (done) return true;
   if (*(volatile int*)fail) return false;
   uint32_t left = kWaitTries;
   asm volatile(
