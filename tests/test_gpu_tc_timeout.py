@@ -49,3 +49,50 @@ def test_expired_waits(kd, impatient, name, batch):  # noqa: F811
         assert (torch.isnan(y) | (y == good)).all()
     again = (kd.matmul_2bit_f16 if name.endswith("f16") else kd.matmul_2bit)(dec, x, xp)
     assert torch.equal(again, good)
+
+
+PROBE = r"""
+#include "kd_tc.cuh"
+__global__ void probe(long long* out) {
+  __shared__ uint64_t bar;
+  __shared__ int fail;
+  if (threadIdx.x == 0) {
+    fail = 0;
+    kd::mbar_init(&bar, 1);
+  }
+  __syncthreads();
+  const long long t0 = clock64();
+  const bool ok = kd::tc_wait(&bar, 0, &fail);  // nothing arrives
+  const long long t1 = clock64();
+  const bool again = kd::tc_wait(&bar, 0, &fail);
+  const long long t2 = clock64();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    out[0] = ok || again;
+    out[1] = fail;
+    out[2] = t1 - t0;
+    out[3] = t2 - t1;
+  }
+}
+extern "C" int run(long long* host) {
+  long long* d;
+  if (cudaMalloc(&d, 32) != cudaSuccess) return 1;
+  probe<<<1, 32>>>(d);
+  const int bad = cudaMemcpy(host, d, 32, cudaMemcpyDeviceToHost) != cudaSuccess;
+  cudaFree(d);
+  return bad;
+}
+"""
+
+
+def test_the_limit_is_a_second(kd, tmp_path):  # noqa: F811
+    """A wait that nothing ends gives up after 0.2 to 3 s of SM cycles at 2 GHz, with the flag
+    set; the next one at once."""
+    from paper_2609_11687_gb300 import build
+    (tmp_path / "probe.cu").write_text(PROBE)
+    so = str(tmp_path / "probe.so")
+    subprocess.run([build._nvcc()] + build.NVCC_FLAGS + ["-shared", "-o", so, str(tmp_path / "probe.cu")], check=True)
+    out = (ctypes.c_longlong * 4)()
+    assert ctypes.CDLL(so).run(out) == 0
+    assert out[0] == 0 and out[1] == 1
+    assert 4e8 <= out[2] <= 6e9 and out[3] <= 1e6, list(out)
