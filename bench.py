@@ -630,8 +630,8 @@ def measure_inference(kd, torch, layer, iters, wss, stream):
                        "achieved": round(deq_bytes / (ms_deq / 1e3) / 1e9, 1), "peak": hbm, "unit": "GB/s",
                        "frac": round(deq_bytes / (ms_deq / 1e3) / 1e9 / hbm, 4), "peak_basis": basis,
                        "algorithmic_bytes_per_param": 4.5},
-        "matmul_2bit": {"kernel": "fold_kernel (1 row) / fold_tc_kernel (2 rows and more: tcgen05, fp32 inputs as three "
-                                  "bf16 pieces; Y = X U_q^T + XP V_q^T from the 2-bit planes: one "
+        "matmul_2bit": {"kernel": "fold_kernel (1 row) / row_grid_kernel and fold_tc_kernel (4 and 16 rows: tcgen05, fp32 inputs "
+                                  "as four bf16 digits on their row's grid; Y = X U_q^T + XP V_q^T from the 2-bit planes: one "
                                   "kd_matmul_2bit_batch per layer; XP by one "
                                   "kd_apply_p_prepared per vector length on tables kd_prepare_p derived once "
                                   "per layer; ms_xp_deriving_tables: kd_apply_p_batch, tables derived per call) "

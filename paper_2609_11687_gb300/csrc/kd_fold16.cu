@@ -7,8 +7,8 @@
 // the rounding of a centre to that type, fp32 accumulation.  Neither plane is expanded
 // in memory.  This file holds the mma.sync kernel for few batch rows, the argument checks and
 // the entry points; the others take kd_fold16_tc.cu, whose tcgen05 form decodes every code once
-// per 256 rows (7B layer: 86 us at 9 rows and 286 us at 512, where 16 rows at a time through
-// mma.sync took 100 us and 3.2 ms; at 8 rows and fewer it is the slower one, 83 against 80 us).
+// per 256 rows (7B layer: 87 us at 9 rows and 280 us at 512, where 16 rows at a time through
+// mma.sync took 100 us and 3.2 ms; at 8 rows and fewer it is the slower one, 83 to 87 against 82 us).
 //
 // Mapping.  mma.m16n8k16 with M = the batch rows (the upper eight only in the form for more than
 // 8 rows), N = 8 output channels, K = 16 inputs: each code becomes its 16-bit centre in registers
@@ -36,7 +36,7 @@ namespace kd {
 namespace {
 
 // Warps of a CTA, which split the inputs: eight (two CTAs per SM), with four the last items
-// of a 7B layer ran on a third of the SMs (86 us per layer at 4 rows, 80 with eight).  Short
+// of a 7B layer ran on a third of the SMs (86 us per layer at 4 rows, 82 with eight).  Short
 // vectors of many channels (wide_short) have four: eight would have one or two groups each and
 // spend their time around them (50257 x 768 at 8 rows: 31 us, 25 with four).
 constexpr int kF16Warps = 8, kF16ShortWarps = 4;

@@ -28,7 +28,7 @@
 // in rank order.  The split follows from the batch alone, so a matrix gives the same bits
 // alone and in a batched call.
 //
-// Measured (7B layer): 84 / 96 / 122 / 155 / 286 us at 9 to 17 / 64 / 128 / 256 / 512 rows; at
+// Measured (7B layer): 87 / 95 / 99 / 117 / 280 us at 9 / 33 / 64 / 129 / 512 rows; at
 // 512 rows that is 1.45 PFLOP/s, 75 % of the measured bf16 rate.  The MMA thread branches on
 // elect.sync (kd_tc.cuh): with a lane test instead, every tcgen05 instruction cost a loop
 // over the lanes and 512 rows took 422 us.

@@ -1,5 +1,5 @@
-// The folded 2-bit layer product of App. C in fp32 (kd_fold.cu states it) on the tensor
-// cores, for two batch rows and more, with nothing rounded to 16 bits.
+// The folded 2-bit layer product of App. C in fp32 (kd_fold.cu states it, and which calls come
+// here) on the tensor cores, with exact sums of the inputs.
 //
 //  * An input is a fixed-point number on the grid of its row (of this CTA's part of it): with
 //    2^k the power of two above the row's largest magnitude, x = 2^k (d1 + d2 + d3 + d4), where
@@ -44,8 +44,9 @@
 // among them (their products with a plain sum could overflow), and rows of more infinities
 // than are noted, are summed again by plain fp32 FMAs.
 //
-// Measured (7B layer, L2 cold): 121 us at 2 rows, 140 at 16, 467 at 64; the table-lookup
-// kernel takes 125 us per two rows (981 at 16).  Error against 64 bits, 2-norm: 5e-8 to 6e-8 (8e-8
+// Measured (7B layer, L2 cold): 119 us at 3 rows, 137 at 16, 454 at 64 (218 and 250 at 3 and 16
+// with centres that are not symmetric); the table-lookup kernel takes 125 us per two rows (981
+// at 16).  The ALU pipe is 64 % busy, mostly with the decode.  Error against 64 bits, 2-norm: 5e-8 to 6e-8 (8e-8
 // with centres that are not symmetric) for normal, all-positive, log-normal and very small inputs
 // and rows led by one, n = 256 to 16384; the table-lookup kernel has 9e-8 to 2.9e-7.
 #include <cuda_runtime.h>
@@ -646,10 +647,10 @@ kd_status fold_tc_run(const kd_fold_mat* mats, int count, int64_t batch, cudaStr
     p.rows = (int)(batch - b0 < kMaxRows ? batch - b0 : kMaxRows);
     p.row_blocks = (p.rows + kRows - 1) / kRows;
     // Up to one row block, two parts per plane: a small layer's tiles alone leave places idle
-    // (16 rows: one 4096 x 11008 matrix 78 -> 44 us, a 768-wide layer's six 27 -> 19), and the
-    // 7B layer takes the same (119 -> 116 us at 2 rows, 130 at 16).  Four parts were slower
-    // (7B layer 159 us at 16 rows), and with more row blocks two already are (17 rows: 222 ->
-    // 238).  Not by the number of tiles: a matrix's results do not depend on the others'.
+    // (16 rows, before the digits: one 4096 x 11008 matrix 78 -> 44 us, a 768-wide layer's six
+    // 27 -> 19), and the 7B layer takes the same (119 -> 116 us at 2 rows, 130 at 16).  Four parts
+    // were slower (7B layer 159 us at 16 rows), and with more row blocks two already are (17
+    // rows: 222 -> 238).  Not by the number of tiles: a matrix's results do not depend on the others'.
     p.split = p.rows <= kRows ? 2 : 1;
     p.count = 0;
     int64_t tiles = 0;
